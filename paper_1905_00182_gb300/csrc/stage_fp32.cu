@@ -1363,7 +1363,7 @@ __global__ void __launch_bounds__(THREADS) k_finish32(Plan p, const float *__res
 }
 
 // 3D viscous term + finish, marching along z.  A 32 x 8 block of threads owns 32 x 8 columns
-// and walks a z-chunk: velocity perturbations of five planes (x, y halo 4) sit in a shared-
+// and walks a z-chunk of zc planes (chosen by march_chunk): velocity perturbations of five planes (x, y halo 4) sit in a shared-
 // memory ring, refilled from registers loaded one plane ahead; at each plane c the 9 gradients
 // are evaluated at the block's cells and at the x/y halo points the x/y divergence needs,
 // giving F_v,x and F_v,y (shared memory, divergence taken at once) and F_v,z, whose
@@ -1373,7 +1373,7 @@ __global__ void __launch_bounds__(THREADS) k_finish32(Plan p, const float *__res
 #define VM_MIN_BLOCKS 4
 #endif
 namespace vm {
-constexpr int TX = 32, TY = 8, ZC = 64;        // block columns, z-chunk
+constexpr int TX = 32, TY = 8;                 // block columns
 constexpr int VT = TX * TY;                    // threads (one column each)
 constexpr int SX = TX + 8, SY = TY + 8;        // staged plane (halo 4)
 constexpr int PX = TX + 4, PY = TY + 4;        // flux points (halo 2)
@@ -1386,15 +1386,15 @@ template <bool STRETCHED>
 __global__ void __launch_bounds__(vm::VT, VM_MIN_BLOCKS) k_visc_march32(Plan p, const float *__restrict__ din,
                                                           float *__restrict__ dout, double *Qn,
                                                           double *__restrict__ Lout, float Bc,
-                                                          float dt, int mode) {
+                                                          float dt, int mode, int zc) {
   using namespace vm;
   extern __shared__ float smm[];
   float *ring = smm;                              // [5][3][SY][SX]
   float *fx = smm + 5 * 3 * SX * SY;              // F_v,x at [TY][PX], 4 components
   float *fy = fx + 4 * PX * TY;                   // F_v,y at [PY][TX], 4 components
   const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
-  const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, zs = blockIdx.z * ZC;
-  const int ze = min(zs + ZC, p.n[2]);
+  const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, zs = blockIdx.z * zc;
+  const int ze = min(zs + zc, p.n[2]);
   const int X = x0 + tx, Y = y0 + ty;
   const bool own = X < p.n[0] && Y < p.n[1];
   Free fs = free_stream(p);
@@ -1768,6 +1768,29 @@ cudaError_t launch_conv(const Plan &p, int first, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+// z-chunk of k_visc_march32.  A block's time is its planes (zc plus ~7 of start-up: the ring's
+// first planes and the two flux planes on each side), whatever its neighbours on the SM do (the
+// pass is bound by latency per plane), so the chunk that minimises (waves of 152 SMs x 4 blocks)
+// x (zc + 7) is taken: long chunks where the columns alone fill the chip, short ones where they
+// do not.  Against a fixed chunk of 64: 99 x 77 x 85 (80 blocks, now 600) 160 -> 45 us, 128^3
+// 176 -> 86 us, 512^3 (chunk 128) 3.80 -> 3.76 ms.
+inline int march_chunk(const int n[3]) {
+  const long long cols =
+      (long long)((n[0] + vm::TX - 1) / vm::TX) * ((n[1] + vm::TY - 1) / vm::TY);
+  const long long slots = 152 * VM_MIN_BLOCKS;
+  int best = 128;
+  long long cost = -1;
+  for (int zc = 128; zc >= 4; zc--) {
+    const long long blocks = cols * ((n[2] + zc - 1) / zc);
+    const long long c = (blocks + slots - 1) / slots * (zc + 7);
+    if (cost < 0 || c < cost) {
+      cost = c;
+      best = zc;
+    }
+  }
+  return best;
+}
+
 template <int DIM, int SCHEME>
 cudaError_t run_stage(const Plan &p, const StageArgs &s, cudaStream_t st) {
   cudaError_t e;
@@ -1836,9 +1859,10 @@ cudaError_t run_stage(const Plan &p, const StageArgs &s, cudaStream_t st) {
     auto kern = stretched ? k_visc_march32<true> : k_visc_march32<false>;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
     if (e != cudaSuccess) return e;
-    dim3 grid((p.n[0] + TX - 1) / TX, (p.n[1] + TY - 1) / TY, (p.n[2] + ZC - 1) / ZC);
+    const int zc = march_chunk(p.n);
+    dim3 grid((p.n[0] + TX - 1) / TX, (p.n[1] + TY - 1) / TY, (p.n[2] + zc - 1) / zc);
     kern<<<grid, VT, SMEM, st>>>(q, din, dout, const_cast<double *>(Qn), s.Lout, (float)s.b,
-                                 (float)s.dt, mode);
+                                 (float)s.dt, mode, zc);
   } else if (p.Re > 0.0)
     k_finish32<DIM, true><<<blocks_for(p.N, THREADS), THREADS, 0, st>>>(
         q, din, dout, const_cast<double *>(Qn), s.Lout, (float)s.b, (float)s.dt, mode);
