@@ -26,6 +26,7 @@
 #include <stdint.h>
 
 #include "ibfsa_internal.h"
+#include "marker.cuh"
 #include "mesh.cuh"
 #include "mlp_tile.cuh"
 #include "tma.cuh"
@@ -1149,117 +1150,70 @@ __device__ __forceinline__ double stage_q(const Plan &p, const double *__restric
   return din ? v + (double)din[c * p.N + o] : v;
 }
 
+// Interpolation (Eq. 8) and penalty force (Eq. 7), one group of lanes per marker (marker.cuh).
 template <int DIM>
-__global__ void k_ib_interp64(Plan p, const double *__restrict__ Qn, const float *__restrict__ din,
-                              const double *__restrict__ xis, const double *xin, double *xio,
-                              double A, double Bc, double dt, int advance) {
-  int k = blockIdx.x * blockDim.x + threadIdx.x;
-  int nm = p.nm, M = p.max_markers;
-  if (k >= nm) return;
-  int j0[3];
-  double w[3][4];
-  if (!point_support<DIM>(p, p.X, M, k, j0, w)) {
-    atomicOr(p.status, IBFSA_STATUS_BOUNDS);
-    for (int a = 0; a < DIM; a++) {
-      p.F[a * M + k] = 0.0;
-      if (advance) xio[a * M + k] = xin[a * M + k];
-    }
-    return;
-  }
-  constexpr int C2 = DIM > 2 ? 4 : 1;
+__global__ void __launch_bounds__(128) k_ib_interp64(Plan p, const double *__restrict__ Qn,
+                                                     const float *__restrict__ din,
+                                                     const double *__restrict__ xis,
+                                                     const double *xin, double *xio, double A,
+                                                     double Bc, double dt, int advance) {
+  constexpr int G = marker::Support<DIM>::G;
+  const int r = threadIdx.x % G, km = (int)((blockIdx.x * blockDim.x + threadIdx.x) / G);
+  const int k = min(km, p.nm - 1);
+  const marker::Support<DIM> t = marker::support<DIM>(p, p.X, p.max_markers, k, r);
   double acc[DIM];
 #pragma unroll
   for (int a = 0; a < DIM; a++) acc[a] = 0.0;
-  for (int r2 = 0; r2 < C2; r2++)
-    for (int r1 = 0; r1 < 4; r1++)
-      for (int r0 = 0; r0 < 4; r0++) {
-        long long o = int_index(p, j0[0] + r0, j0[1] + r1, j0[2] + r2);
-        double wt = w[0][r0] * w[1][r1] * w[2][r2];
-        double inv_rho = 1.0 / stage_q(p, Qn, din, 0, o);
+  if (t.ok) {
+    const long long o = int_index(p, t.j0[0], t.j0[1] + (r & 3), t.j0[2] + (r >> 2));
 #pragma unroll
-        for (int a = 0; a < DIM; a++) acc[a] += stage_q(p, Qn, din, 1 + a, o) * inv_rho * wt;
-      }
+    for (int r0 = 0; r0 < 4; r0++) {
+      const double wi = t.w0[r0] * (1.0 / stage_q(p, Qn, din, 0, o + r0));
 #pragma unroll
-  for (int a = 0; a < DIM; a++) {
-    double slip = acc[a] - p.U[a * M + k];
-    p.F[a * M + k] = p.alpha_pen * xis[a * M + k] + p.beta_pen * slip;
-    if (advance) xio[a * M + k] = A * xin[a * M + k] + Bc * (xis[a * M + k] + dt * slip);
+      for (int a = 0; a < DIM; a++) acc[a] = fma(stage_q(p, Qn, din, 1 + a, o + r0), wi, acc[a]);
+    }
   }
+#pragma unroll
+  for (int a = 0; a < DIM; a++) acc[a] = marker::group_sum<DIM>(acc[a] * t.wr);
+  if (km >= p.nm) return;
+  if (t.ok) marker::force<DIM>(p, k, r, acc, xis, xin, xio, A, Bc, dt, advance);
+  else marker::off_grid<DIM>(p, k, r, xin, xio, advance);
 }
 
-// Spreading (Eq. 9) into the FP32 right-hand side: one group of S = 4^DIM threads per marker,
-// one thread per support cell.  The marker's 4 DIM kernel weights (FP64, Eq. 11) are evaluated
-// once, by the first 4 DIM threads of its group, and shared; the per-cell force, the fluid
-// velocity of the power term f.u and the atomic additions are FP32, the precision of the
-// right-hand side they enter.
+// Spreading (Eq. 9) into the FP32 right-hand side, one group of lanes per marker (marker.cuh),
+// four support cells per lane.  The kernel weights and the marker's force are FP64; the per-cell
+// force, the fluid velocity of the power term f.u and the atomic additions are FP32, the
+// precision of the right-hand side they enter.
 template <int DIM>
 __global__ void __launch_bounds__(128) k_spread32(Plan p, const double *__restrict__ Qn,
                                                   const float *__restrict__ din) {
-  constexpr int S = DIM > 2 ? 64 : 16, MPB = 128 / S;
-  __shared__ double sw[MPB][3][4];
-  __shared__ int sj[MPB][3];
-  __shared__ float sf[MPB][3];
-  __shared__ int sok[MPB];
-  const int lm = threadIdx.x / S, r = threadIdx.x % S;
-  const int k = blockIdx.x * MPB + lm;
-  const int M = p.max_markers;
-  const bool live = k < p.nm;
-  const bool stretched = p.mx[0] || p.mx[1] || p.mx[2];
-  if (live && r < 4 * DIM && !stretched) {
-    int a = r / 4, q = r % 4;
-    double s = (p.X[a * M + k] - p.lo[a]) * p.inv_h[a] - 0.5;
-    int j0 = (int)floor(s) - 1;
-    sw[lm][a][q] = peskin(s - (double)(j0 + q));
-    if (q == 0) sj[lm][a] = j0;
-  }
-  if (live && r == 0) {
-    bool ok = true;
-    double hprod = p.hprod;
-    if (stretched) {  // one thread finds the marker's supports and its local spacings
-      int j0[3];
-      double w[3][4];
-      ok = point_support<DIM>(p, p.X, M, k, j0, w, &hprod);
+  constexpr int G = marker::Support<DIM>::G;
+  const int r = threadIdx.x % G, km = (int)((blockIdx.x * blockDim.x + threadIdx.x) / G);
+  const int k = min(km, p.nm - 1), M = p.max_markers;
+  const marker::Support<DIM> t = marker::support<DIM>(p, p.X, M, k, r);
+  if (km >= p.nm || !t.ok) return;  // the interpolation kernel reports markers off the grid
+  const double sc = p.dS[k] * t.ihp;
+  float f[DIM];
 #pragma unroll
-      for (int a = 0; a < DIM; a++) {
-        sj[lm][a] = j0[a];
+  for (int a = 0; a < DIM; a++) f[a] = (float)(-p.F[a * M + k] * sc);
+  const Free fs = free_stream(p);
+  const long long o = int_index(p, t.j0[0], t.j0[1] + (r & 3), t.j0[2] + (r >> 2));
 #pragma unroll
-        for (int q = 0; q < 4; q++) sw[lm][a][q] = w[a][q];
-      }
-    } else {
+  for (int r0 = 0; r0 < 4; r0++) {
+    const float wt = (float)(t.w0[r0] * t.wr);
+    const float d0 = p.qn32[o + r0] + (din ? din[o + r0] : 0.f);
+    const float inv_rho = 1.f / (fs.rho + d0);
+    float pw = 0.f;
 #pragma unroll
-      for (int a = 0; a < DIM; a++) {
-        double s = (p.X[a * M + k] - p.lo[a]) * p.inv_h[a] - 0.5;
-        int j0 = (int)floor(s) - 1;
-        if (j0 < 0 || j0 + 3 > p.n[a] - 1) ok = false;
-      }
+    for (int a = 0; a < DIM; a++) {
+      const long long at = (1 + a) * p.N + o + r0;
+      const float da = p.qn32[at] + (din ? din[at] : 0.f);
+      const float fa = f[a] * wt;
+      atomicAdd(&p.L32[at], fa);
+      pw += fa * ((fs.m[a] + da) * inv_rho);
     }
-    sok[lm] = ok;
-    double sc = p.dS[k] / hprod;
-#pragma unroll
-    for (int a = 0; a < 3; a++) sf[lm][a] = a < DIM ? (float)(-p.F[a * M + k] * sc) : 0.f;
-    if (DIM < 3) {
-      sw[lm][2][0] = 1.0;
-      sw[lm][2][1] = sw[lm][2][2] = sw[lm][2][3] = 0.0;
-      sj[lm][2] = 0;
-    }
+    atomicAdd(&p.L32[(DIM + 1) * p.N + o + r0], pw);
   }
-  __syncthreads();
-  if (!live || !sok[lm]) return;  // the interpolation kernel reports markers off the grid
-  int r0 = r & 3, r1 = (r >> 2) & 3, r2 = DIM > 2 ? (r >> 4) : 0;
-  float wt = (float)(sw[lm][0][r0] * sw[lm][1][r1] * sw[lm][2][r2]);
-  long long o = int_index(p, sj[lm][0] + r0, sj[lm][1] + r1, sj[lm][2] + r2);
-  Free fs = free_stream(p);
-  float d0 = p.qn32[o] + (din ? din[o] : 0.f);
-  float inv_rho = 1.f / (fs.rho + d0);
-  float pw = 0.f;
-#pragma unroll
-  for (int a = 0; a < DIM; a++) {
-    float da = p.qn32[(1 + a) * p.N + o] + (din ? din[(1 + a) * p.N + o] : 0.f);
-    float fa = sf[lm][a] * wt;
-    atomicAdd(&p.L32[(1 + a) * p.N + o], fa);
-    pw += fa * ((fs.m[a] + da) * inv_rho);
-  }
-  atomicAdd(&p.L32[(DIM + 1) * p.N + o], pw);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1808,8 +1762,8 @@ cudaError_t run_stage(const Plan &p, const StageArgs &s, cudaStream_t st) {
   int advance = s.stage >= 0;
   if (p.nm > 0) {
     prof_begin(pr, st);
-    k_ib_interp64<DIM><<<blocks_for(p.nm, 128), 128, 0, st>>>(p, Qn, din, s.xis, s.xin, s.xio,
-                                                             s.a, s.b, s.dt, advance);
+    k_ib_interp64<DIM><<<blocks_for((long long)p.nm * marker::Support<DIM>::G, 128), 128, 0, st>>>(
+        p, Qn, din, s.xis, s.xin, s.xio, s.a, s.b, s.dt, advance);
     prof_end(pr, K_INTERP, st);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
@@ -1843,9 +1797,9 @@ cudaError_t run_stage(const Plan &p, const StageArgs &s, cudaStream_t st) {
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   if (p.nm > 0) {
-    constexpr int MPB = DIM > 2 ? 2 : 8;  // markers per 128-thread block
     prof_begin(pr, st);
-    k_spread32<DIM><<<blocks_for(p.nm, MPB), 128, 0, st>>>(p, Qn, din);
+    k_spread32<DIM><<<blocks_for((long long)p.nm * marker::Support<DIM>::G, 128), 128, 0, st>>>(
+        p, Qn, din);
     prof_end(pr, K_SPREAD, st);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }

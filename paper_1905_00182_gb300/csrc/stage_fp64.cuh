@@ -14,6 +14,7 @@
 #include <stdint.h>
 
 #include "ibfsa_internal.h"
+#include "marker.cuh"
 #include "mesh.cuh"
 
 #ifndef IBFSA_STRICT
@@ -803,6 +804,29 @@ __global__ void k_ib_interp(Plan p, const double *__restrict__ xis, const double
                             double *xio, double A, double Bc, double dt, int advance) {
   int k = blockIdx.x * blockDim.x + threadIdx.x;
   int nm = p.nm, M = p.max_markers;
+  if constexpr (!STRICT) {  // one group of lanes per marker (marker.cuh)
+    constexpr int G = marker::Support<DIM>::G;
+    const int r = threadIdx.x % G, km = (int)((blockIdx.x * blockDim.x + threadIdx.x) / G);
+    k = min(km, nm - 1);
+    const marker::Support<DIM> t = marker::support<DIM>(p, p.X, M, k, r);
+    double acc[DIM];
+#pragma unroll
+    for (int a = 0; a < DIM; a++) acc[a] = 0.0;
+    if (t.ok) {
+      const long long s = pad_index(p, t.j0[0], t.j0[1] + (r & 3), t.j0[2] + (r >> 2));
+#pragma unroll
+      for (int a = 0; a < DIM; a++)
+#pragma unroll
+        for (int r0 = 0; r0 < 4; r0++) acc[a] = fma(p.Wp[a * p.NP + s + r0], t.w0[r0], acc[a]);
+    }
+#pragma unroll
+    for (int a = 0; a < DIM; a++) acc[a] = marker::group_sum<DIM>(acc[a] * t.wr);
+    if (km >= nm) return;
+    if (t.ok) marker::force<DIM>(p, k, r, acc, xis, xin, xio, A, Bc, dt, advance);
+    else marker::off_grid<DIM>(p, k, r, xin, xio, advance);
+    return;
+  }
+  // strict: one thread per marker, in the order of the formulas
   if (k >= nm) return;
   int j0[3];
   double w[3][4];
@@ -856,31 +880,32 @@ __global__ void k_spread_ordered(Plan p) {
   }
 }
 
-// fast spreading: one thread per (marker, support cell), atomics straight into L:
-// momentum += f, energy += f.u
+// fast spreading: one group of lanes per marker, four support cells per lane (marker.cuh),
+// atomics straight into L: momentum += f, energy += f.u
 template <int DIM>
-__global__ void k_spread_atomic(Plan p) {
-  constexpr int S = DIM > 2 ? 64 : 16;
-  long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (long long)p.nm * S) return;
-  int k = (int)(t / S), r = (int)(t % S);
-  int r0 = r & 3, r1 = (r >> 2) & 3, r2 = DIM > 2 ? (r >> 4) : 0;
-  int M = p.max_markers;
-  int j0[3];
-  double w[3][4], hprod;
-  if (!marker_support<DIM>(p, p.X, M, k, j0, w, &hprod)) return;
-  double wt = w[0][r0] * w[1][r1] * w[2][r2];
-  long long o = int_index(p, j0[0] + r0, j0[1] + r1, j0[2] + r2);
-  long long s = pad_index(p, j0[0] + r0, j0[1] + r1, j0[2] + r2);
-  double scale = wt * p.dS[k] / hprod;
-  double pw = 0.0;
+__global__ void __launch_bounds__(128) k_spread_atomic(Plan p) {
+  constexpr int G = marker::Support<DIM>::G;
+  const int r = threadIdx.x % G, km = (int)((blockIdx.x * blockDim.x + threadIdx.x) / G);
+  const int k = min(km, p.nm - 1), M = p.max_markers;
+  const marker::Support<DIM> t = marker::support<DIM>(p, p.X, M, k, r);
+  if (km >= p.nm || !t.ok) return;
+  const long long o = int_index(p, t.j0[0], t.j0[1] + (r & 3), t.j0[2] + (r >> 2));
+  const long long s = pad_index(p, t.j0[0], t.j0[1] + (r & 3), t.j0[2] + (r >> 2));
+  const double sc = t.wr * (p.dS[k] * t.ihp);
+  double f[DIM];
 #pragma unroll
-  for (int a = 0; a < DIM; a++) {
-    double fa = -p.F[a * M + k] * scale;
-    atomicAdd(&p.L[(1 + a) * p.N + o], fa);
-    pw += fa * p.Wp[a * p.NP + s];
+  for (int a = 0; a < DIM; a++) f[a] = -p.F[a * M + k] * sc;
+#pragma unroll
+  for (int r0 = 0; r0 < 4; r0++) {
+    double pw = 0.0;
+#pragma unroll
+    for (int a = 0; a < DIM; a++) {
+      const double fa = f[a] * t.w0[r0];
+      atomicAdd(&p.L[(1 + a) * p.N + o + r0], fa);
+      pw += fa * p.Wp[a * p.NP + s + r0];
+    }
+    atomicAdd(&p.L[(DIM + 1) * p.N + o + r0], pw);
   }
-  atomicAdd(&p.L[(DIM + 1) * p.N + o], pw);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1023,8 +1048,9 @@ cudaError_t run_stage(const Plan &p, const StageArgs &s, cudaStream_t st) {
   int advance = s.stage >= 0;
   if (p.nm > 0) {
     prof_begin(pr, st);
-    k_ib_interp<DIM><<<blocks_for(p.nm, 128), 128, 0, st>>>(p, s.xis, s.xin, s.xio, s.a, s.b,
-                                                           s.dt, advance);
+    const long long lanes = (long long)p.nm * (STRICT ? 1 : marker::Support<DIM>::G);
+    k_ib_interp<DIM><<<blocks_for(lanes, 128), 128, 0, st>>>(p, s.xis, s.xin, s.xio, s.a, s.b,
+                                                             s.dt, advance);
     prof_end(pr, K_INTERP, st);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
@@ -1070,9 +1096,9 @@ cudaError_t run_stage(const Plan &p, const StageArgs &s, cudaStream_t st) {
       k_spread_ordered<DIM><<<1, DIM > 2 ? 64 : 16, 0, st>>>(p);
       prof_end(pr, K_SPREAD, st);
     } else {
-      constexpr int S = DIM > 2 ? 64 : 16;
       prof_begin(pr, st);
-      k_spread_atomic<DIM><<<blocks_for((long long)p.nm * S, THREADS), THREADS, 0, st>>>(p);
+      k_spread_atomic<DIM><<<blocks_for((long long)p.nm * marker::Support<DIM>::G, 128), 128, 0,
+                             st>>>(p);
       prof_end(pr, K_SPREAD, st);
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
