@@ -30,9 +30,36 @@ constexpr int THREADS = 256;
 // ------------------------------------------------------------------------------------------
 // small helpers
 // ------------------------------------------------------------------------------------------
+// x / d given inv_d = 1/d correctly rounded.  Strict: the correctly rounded quotient without the
+// divider, by Markstein's theorem: from a q within an ulp of x/d, RN(q + inv_d RN(x - d q)) is
+// x/d correctly rounded (the remainder is exact, its product a correction far below an ulp).  One
+// such step brings x inv_d within an ulp of x/d, the second rounds it: 5 FP64 operations against
+// ~9.  The divider outside the exponents where nothing over- or underflows on the way.
 __device__ __forceinline__ double divide(double x, double d, double inv_d) {
-  if constexpr (STRICT) return x / d;
-  else return x * inv_d;
+  if constexpr (STRICT) {
+    const unsigned ex = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
+    const unsigned ed = ((unsigned)__double2hiint(d) >> 20) & 0x7ffu;
+    if (ex - 600u < 900u && ed - 723u < 600u) {
+      double q = x * inv_d;
+      q = __fma_rn(__fma_rn(-d, q, x), inv_d, q);
+      return __fma_rn(__fma_rn(-d, q, x), inv_d, q);
+    }
+    return x == 0.0 && ed - 723u < 600u ? x * inv_d : x / d;
+  } else {
+    return x * inv_d;
+  }
+}
+
+// x / 6 in the same way; the rounded sixth is within a quarter of an ulp (2^-54 relative), so the
+// product is already within an ulp and one step rounds it: 3 operations
+__device__ __forceinline__ double divide6(double x) {
+  const double r = 1.0 / 6.0;
+  const unsigned ex = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
+  if (ex - 600u < 900u) {
+    const double q = x * r;
+    return __fma_rn(__fma_rn(-6.0, q, x), r, q);
+  }
+  return x == 0.0 ? x * r : x / 6.0;
 }
 
 // ghost rule of one direction: interior index, or -1 for a free-stream ghost
@@ -138,9 +165,7 @@ __device__ __forceinline__ double weno5js(double a, double b, double c, double d
 
 // TENO5: gamma_k = (1 + tau5/(beta_k + 1e-40))^6, tau5 = |beta_0 - beta_2|; stencil k kept when
 // gamma_k / sum gamma >= 1e-5; omega = normalised linear weights of the kept stencils
-__device__ __forceinline__ double teno5(const Plan &p, double a, double b, double c, double d,
-                                        double e) {
-  Cands k = candidates(a, b, c, d, e);
+__device__ __forceinline__ int teno_keep(const Cands &k) {
   const double eps = 1e-40, CT = 1e-5;
   double tau5 = fabs(k.b0 - k.b2);
   double g0, g1, g2;
@@ -162,47 +187,192 @@ __device__ __forceinline__ double teno5(const Plan &p, double a, double b, doubl
     double th = CT * (g0 + g1 + g2);
     mask = (g0 >= th ? 1 : 0) | (g1 >= th ? 2 : 0) | (g2 >= th ? 4 : 0);
   }
-  const double *w = p.teno_w[mask];
+  return mask;
+}
+
+__device__ __forceinline__ double teno5(const Plan &p, double a, double b, double c, double d,
+                                        double e) {
+  const Cands k = candidates(a, b, c, d, e);
+  const double *w = p.teno_w[teno_keep(k)];
   return w[0] * k.q0 + w[1] * k.q1 + w[2] * k.q2;
 }
 
-// Fast arithmetic only: TENO5 keeps every stencil when tau5 <= 4 (min beta + eps) -- each
-// gamma_k lies in [1, 5^6], so chi_k >= 1/(3 5^6) = 2.1e-5 > C_T -- and the reconstruction is
-// the optimal linear combination (2a - 13b + 47c + 27d - 3e)/60 (the strict form evaluates
-// every step as written).  Only this sufficient test is taken in FP32 (the FP64 pipe is the
-// bound; a conversion issues at the FP64 rate): the four first differences in FP64, rounded to
-// FP32, give t and u of every indicator (t0 = d2 - d1, u0 = 3 d2 - d1, t1 = d3 - d2,
-// u1 = -(d2 + d3), t2 = d4 - d3, u2 = d4 - 3 d3), taken times 4, (13/3) t^2 + u^2, against
-// 4 min + 1.6e-29.  Each indicator is a positive definite form of its two differences, so its
-// relative error stays a few 1e-7 (where t or u cancels, the other term dominates) -- far
-// inside the test's factor-2 margin in chi_k (2.1e-5 against C_T = 1e-5): a stencil the test
-// keeps is one TENO5 keeps; where the test fails, the full FP64 TENO5 decides.  Differences
-// below FP32's range flush to zero and pass the test; their stencils vary by less than 1e-17
-// of the flux, whatever TENO5 would cut.
-__device__ __forceinline__ double teno5_fast(const Plan &p, double a, double b, double c,
-                                             double d, double e) {
-  const double e1 = b - a, e2 = c - b, e3 = d - c, e4 = e - d;
-  const float d1 = (float)e1, d2 = (float)e2, d3 = (float)e3, d4 = (float)e4;
-  const float t0 = d2 - d1, u0 = fmaf(3.f, d2, -d1);
-  const float t1 = d3 - d2, u1 = d2 + d3;
-  const float t2 = d4 - d3, u2 = fmaf(-3.f, d3, d4);
-  const float k13 = 13.f / 3.f;
-  const float b0 = fmaf(k13 * t0, t0, u0 * u0);
-  const float b1 = fmaf(k13 * t1, t1, u1 * u1);
-  const float b2 = fmaf(k13 * t2, t2, u2 * u2);
-  // the linear combination as c plus its differences, (-2 d1 + 11 d2 + 24 d3 - 3 d4)/60: four
-  // fused multiply-adds, and a constant stencil gives c exactly
-  if (fabsf(b0 - b2) <= fmaf(4.f, fminf(b0, fminf(b1, b2)), 1.6e-29f))
-    return fma(-3.0 / 60.0, e4, fma(24.0 / 60.0, e3, fma(11.0 / 60.0, e2, fma(-2.0 / 60.0, e1, c))));
-  return teno5(p, a, b, c, d, e);
+// An FP64 value as FP32 by integer operations, truncated: a conversion instruction issues at the
+// FP64 rate (1.8 per clock and SM), these at the integer rate.  Magnitudes below FP32's normal
+// range give 0, above it (and non-finite values) NaN.
+__device__ __forceinline__ float low_precision(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned e = hi & 0x7ff00000u;
+  unsigned r = ((__funnelshift_l(lo, hi, 3) & 0x7fffffffu) ^ 0x40000000u) | (hi & 0x80000000u);
+  r = e < 0x38100000u ? 0u : r;
+  r = e >= 0x47f00000u ? 0x7fffffffu : r;
+  return __uint_as_float(r);
+}
+
+// TENO5 keeps every stencil when tau5 <= 4 (min beta + eps) -- each gamma_k lies in [1, 5^6], so
+// chi_k >= 1/(3 5^6) = 2.1e-5 > C_T -- and its weights are then the linear ones.  Only this
+// sufficient test is taken in FP32 (the FP64 pipe is the bound), from the stencil's four FP64
+// first differences d: t0 = d1 - d0, u0 = 3 d1 - d0, t1 = d2 - d1, u1 = d1 + d2, t2 = d3 - d2,
+// u2 = d3 - 3 d2, indicators times 4, kt_k = (13/3) t_k^2 plus u_k^2.  Each indicator is a
+// positive definite form of its two differences, so its relative error stays a few 1e-7 (where t
+// or u cancels, the other term dominates) -- far inside the test's factor-2 margin in chi_k: a
+// stencil the test keeps is one TENO5 keeps; where the test fails (or anything is not finite),
+// the FP64 TENO5 decides.  Reversing the stencil swaps the outer indicators and leaves the test.
+// Fast form: differences below FP32's range flush to zero and pass; their stencils vary by less
+// than 1e-17 of the flux, whatever TENO5 would cut.  Strict form: its indicators carry the
+// rounding of a - 4b + 3c and the like, up to 1e-15 |f| in their square roots, so the test passes
+// only where the smallest is at least (2e-13 c)^2 (c the stencil's middle value; an indicator is
+// at least 0.98 of its squared differences, so values much larger than c imply a larger one) and
+// well inside FP32's range.
+__device__ __forceinline__ bool all_kept(float d0, float d1, float d2, float d3, float kt0,
+                                         float kt1, float kt2, double c) {
+  const float u0 = fmaf(3.f, d1, -d0), u1 = d1 + d2, u2 = fmaf(-3.f, d2, d3);
+  const float b0 = fmaf(u0, u0, kt0), b1 = fmaf(u1, u1, kt1), b2 = fmaf(u2, u2, kt2);
+  const float m = fminf(b0, fminf(b1, b2));
+  if constexpr (STRICT)
+    return fabsf(b0 - b2) <= 4.f * m &&
+           m >= fmaxf(1e-35f, 4e-26f * low_precision(c) * low_precision(c));
+  else
+    return fabsf(b0 - b2) <= fmaf(4.f, m, 1.6e-29f);
+}
+
+// Strict form, constant stencil (quiescent fluid): every difference and the first two indicators
+// are exactly zero; the third carries the rounding of 3c, r = (3c - 4c) + c, beta2 = r^2 / 4.
+// r = 0: all stencils kept (7).  |r| > 1e-18: tau5 / (0 + 1e-40) > 2000, so the third stencil's
+// weight, at most 64 of 2 (2000)^6, is cut and the others' are near a half (3).  Otherwise, or if
+// the stencil is not constant: -1.
+__device__ __forceinline__ int constant_mask(double d0, double d1, double d2, double d3, double c) {
+  const unsigned long long any =
+      (unsigned long long)(__double_as_longlong(d0) | __double_as_longlong(d1) |
+                           __double_as_longlong(d2) | __double_as_longlong(d3));
+  if (any << 1) return -1;
+  const double r = 3.0 * c - 4.0 * c + c;
+  return r == 0.0 ? 7 : fabs(r) > 1e-18 ? 3 : -1;
+}
+
+// Reconstruction at K consecutive faces of one line from one side's split fluxes f[0 .. K+3]
+// (in increasing cell index): face j from f[j .. j+4], upwind to downwind (REV: downwind to
+// upwind).  What neighbouring faces share is taken once: first differences, second differences
+// and their squares.  Of the 12 FP64 operations a TENO5 face took by itself (four differences,
+// four conversions, four fused multiply-adds) 4 + (K + 3)/K remain; WENO5-JS goes from 62 to 38.
+// strict: every value the oracle computes is computed by the same roundings, once instead of for
+// each face that uses it, and TENO5's weights are looked up without its divisions where the
+// sufficient test above proves that it keeps every stencil.  Returns the faces (bit j) whose
+// stencil neither passes that test nor is constant: the caller replaces their h by teno5.
+template <int SCHEME, bool REV, int K>
+__device__ __forceinline__ unsigned faces_of_line(const Plan &p, const double (&f)[K + 4],
+                                                  double (&h)[K]) {
+  unsigned fail = 0;
+  if constexpr (SCHEME == IBFSA_TENO5) {
+    double d[K + 3];
+    float s[K + 3], kt[K + 2];
+#pragma unroll
+    for (int j = 0; j < K + 3; j++) {
+      d[j] = f[j + 1] - f[j];
+      s[j] = low_precision(d[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < K + 2; j++) {
+      const float t = s[j + 1] - s[j];
+      kt[j] = (13.f / 3.f) * t * t;
+    }
+#pragma unroll
+    for (int j = 0; j < K; j++) {
+      const double a = f[REV ? j + 4 : j], b = f[REV ? j + 3 : j + 1], c = f[j + 2];
+      const double dd = f[REV ? j + 1 : j + 3], e = f[REV ? j : j + 4];
+      const bool keep = all_kept(s[j], s[j + 1], s[j + 2], s[j + 3], kt[j], kt[j + 1], kt[j + 2], c);
+      if constexpr (STRICT) {
+        int mask = 7;
+        if (!keep) {
+          mask = constant_mask(d[j], d[j + 1], d[j + 2], d[j + 3], c);
+          if (mask < 0) fail |= 1u << j;
+        }
+        const double *w = p.teno_w[mask & 7];
+        const double q0 = divide6(2.0 * a - 7.0 * b + 11.0 * c);
+        const double q1 = divide6(-b + 5.0 * c + 2.0 * dd);
+        const double q2 = divide6(2.0 * c + 5.0 * dd - e);
+        h[j] = w[0] * q0 + w[1] * q1 + w[2] * q2;
+      } else {
+        if (!keep) fail |= 1u << j;
+        // the linear combination (2a - 13b + 47c + 27d - 3e)/60 as c plus its differences: four
+        // fused multiply-adds, and a constant stencil gives c exactly
+        const double sg = REV ? -1.0 : 1.0;
+        const double e1 = d[REV ? j + 3 : j], e2 = d[REV ? j + 2 : j + 1];
+        const double e3 = d[REV ? j + 1 : j + 2], e4 = d[REV ? j : j + 3];
+        h[j] = fma(sg * -3.0 / 60.0, e4,
+                   fma(sg * 24.0 / 60.0, e3, fma(sg * 11.0 / 60.0, e2, fma(sg * -2.0 / 60.0, e1, c))));
+      }
+    }
+  } else if constexpr (STRICT) {
+    // kt[j] of the triple f[j], f[j+1], f[j+2], its second difference rounded in the order the
+    // stencil's direction gives
+    double kt[K + 2];
+#pragma unroll
+    for (int j = 0; j < K + 2; j++) {
+      const double t = REV ? f[j + 2] - 2.0 * f[j + 1] + f[j] : f[j] - 2.0 * f[j + 1] + f[j + 2];
+      kt[j] = 13.0 / 12.0 * t * t;
+    }
+#pragma unroll
+    for (int j = 0; j < K; j++) {
+      const double a = f[REV ? j + 4 : j], b = f[REV ? j + 3 : j + 1], c = f[j + 2];
+      const double d = f[REV ? j + 1 : j + 3], e = f[REV ? j : j + 4];
+      const double eps = 1e-6;
+      double t;
+      t = a - 4.0 * b + 3.0 * c;
+      const double b0 = kt[REV ? j + 2 : j] + 0.25 * t * t;
+      t = b - d;
+      const double b1 = kt[j + 1] + 0.25 * t * t;
+      t = 3.0 * c - 4.0 * d + e;
+      const double b2 = kt[REV ? j : j + 2] + 0.25 * t * t;
+      const double al0 = 0.1 / ((eps + b0) * (eps + b0));
+      const double al1 = 0.6 / ((eps + b1) * (eps + b1));
+      const double al2 = 0.3 / ((eps + b2) * (eps + b2));
+      const double s = al0 + al1 + al2;
+      h[j] = (al0 / s) * divide6(2.0 * a - 7.0 * b + 11.0 * c) +
+             (al1 / s) * divide6(-b + 5.0 * c + 2.0 * d) + (al2 / s) * divide6(2.0 * c + 5.0 * d - e);
+    }
+  } else {
+    // S_k = 4 (eps + beta_k), weights d_k / S_k^2 over their common denominator, the
+    // reconstruction as c plus a weighted mean of the candidates' differences from c
+    double d[K + 3], kt[K + 2];
+#pragma unroll
+    for (int j = 0; j < K + 3; j++) d[j] = f[j + 1] - f[j];
+#pragma unroll
+    for (int j = 0; j < K + 2; j++) {
+      const double t = d[j + 1] - d[j];
+      kt[j] = fma(13.0 / 3.0 * t, t, 4e-6);
+    }
+#pragma unroll
+    for (int j = 0; j < K; j++) {
+      const double sg = REV ? -1.0 : 1.0;
+      const double e1 = sg * d[REV ? j + 3 : j], e2 = sg * d[REV ? j + 2 : j + 1];
+      const double e3 = sg * d[REV ? j + 1 : j + 2], e4 = sg * d[REV ? j : j + 3];
+      const double u0 = fma(3.0, e2, -e1), u1 = e2 + e3, u2 = fma(-3.0, e3, e4);
+      double s0 = fma(u0, u0, kt[REV ? j + 2 : j]), s1 = fma(u1, u1, kt[j + 1]);
+      double s2 = fma(u2, u2, kt[REV ? j : j + 2]);
+      s0 *= s0;
+      s1 *= s1;
+      s2 *= s2;
+      const double p0 = s1 * s2, p1 = s0 * s2, p2 = s0 * s1;  // weights p0 : 6 p1 : 3 p2
+      const double x3 = 12.0 * e3;
+      const double n0 = fma(5.0, e2, -2.0 * e1), n1 = fma(6.0, e2, x3), n2 = fma(-3.0, e4, x3);
+      const double num = fma(p2, n2, fma(p1, n1, p0 * n0));  // 6 (candidate - c), weighted
+      const double den = fma(18.0, p2, fma(36.0, p1, 6.0 * p0));
+      h[j] = f[j + 2] + num / den;
+    }
+  }
+  return fail;
 }
 
 template <int SCHEME>
 __device__ __forceinline__ double recon(const Plan &p, double a, double b, double c, double d,
                                         double e) {
-  if constexpr (SCHEME == IBFSA_TENO5) {
-    if constexpr (STRICT) return teno5(p, a, b, c, d, e);
-    else return teno5_fast(p, a, b, c, d, e);
+  if constexpr (SCHEME == IBFSA_TENO5 && !STRICT) {
+    const double f[5] = {a, b, c, d, e};
+    double h[1];
+    return faces_of_line<IBFSA_TENO5, false, 1>(p, f, h) ? teno5(p, a, b, c, d, e) : h[0];
+  } else if constexpr (SCHEME == IBFSA_TENO5) {
+    return teno5(p, a, b, c, d, e);
   } else {
     return weno5js(a, b, c, d, e);
   }
@@ -249,11 +419,11 @@ __global__ void __launch_bounds__(THREADS) k_pad(Plan p, const double *__restric
     for (int c = 0; c < NV; c++) p.Qp[c * p.NP + t] = q[c];
     double rho = q[0];
     double ke = 0.0, u[DIM];
-    // strict: each division as the oracle writes it; fast: one reciprocal of rho
-    const double inv_rho = STRICT ? 0.0 : 1.0 / rho;
+    // one reciprocal of rho (strict: the quotients rounded as divisions, see divide)
+    const double inv_rho = 1.0 / rho;
 #pragma unroll
     for (int a = 0; a < DIM; a++) {
-      u[a] = STRICT ? q[1 + a] / rho : q[1 + a] * inv_rho;
+      u[a] = divide(q[1 + a], rho, inv_rho);
       ke += q[1 + a] * u[a];
       p.Wp[a * p.NP + t] = u[a];
     }
@@ -261,7 +431,7 @@ __global__ void __launch_bounds__(THREADS) k_pad(Plan p, const double *__restric
     p.Wp[DIM * p.NP + t] = pr;
     if (interior) {
       if constexpr (STRICT) {
-        const double c = sqrt(p.gamma * pr / rho);
+        const double c = sqrt(divide(p.gamma * pr, rho, inv_rho));
 #pragma unroll
         for (int a = 0; a < DIM; a++) wmax[a] = fabs(u[a]) + c;
       } else {
@@ -325,8 +495,7 @@ __global__ void __launch_bounds__(THREADS) k_pad(Plan p, const double *__restric
 }
 
 // ------------------------------------------------------------------------------------------
-// convective term along direction A: split fluxes of a tile of lines staged in shared memory,
-// one face per thread per pass, conservative difference into L
+// convective term along direction A
 // ------------------------------------------------------------------------------------------
 // ------------------------------------------------------------------------------------------
 // characteristic-wise option: eigenvectors of the Euler flux Jacobian along A at the Roe
@@ -420,13 +589,11 @@ __host__ __device__ constexpr size_t conv_smem_bytes() {
   return sizeof(double) * 2 * (DIM + 2) * ConvTile<A>::ROWS * ConvTile<A>::LEN;
 }
 
-template <int DIM, int A, int SCHEME, bool CHAR>
-__global__ void __launch_bounds__(THREADS) k_conv(Plan p, int first) {
+// characteristic-wise: split fluxes of a tile of lines staged in shared memory, one face per
+// thread per pass, conservative difference into L
+template <int DIM, int A, int SCHEME>
+__global__ void __launch_bounds__(THREADS) k_conv_char(Plan p, int first) {
   constexpr int NV = DIM + 2;
-  // TENO5's weights depend on ratios of indicators only (its floors aside), so its fast
-  // component-wise form can reconstruct F +- alpha q and halve once at the face; WENO5-JS's
-  // eps = 1e-6 is not scale-free
-  constexpr bool FOLD = !STRICT && !CHAR && SCHEME == IBFSA_TENO5;
   using T = ConvTile<A>;
   extern __shared__ double sm[];
   double *sfp = sm;                              // [NV][ROWS][LEN]
@@ -485,9 +652,8 @@ __global__ void __launch_bounds__(THREADS) k_conv(Plan p, int first) {
           F = q * ua;
           if (c - 1 == A) F += pr;
         }
-        // fast component-wise TENO5: F +- alpha q, the halves taken once at the face
-        sfp[(c * T::ROWS + row) * T::LEN + l] = FOLD ? fma(alpha, q, F) : 0.5 * (F + alpha * q);
-        sfm[(c * T::ROWS + row) * T::LEN + l] = FOLD ? fma(-alpha, q, F) : 0.5 * (F - alpha * q);
+        sfp[(c * T::ROWS + row) * T::LEN + l] = 0.5 * (F + alpha * q);
+        sfm[(c * T::ROWS + row) * T::LEN + l] = 0.5 * (F - alpha * q);
       }
     } else {
 #pragma unroll
@@ -510,63 +676,52 @@ __global__ void __launch_bounds__(THREADS) k_conv(Plan p, int first) {
       else { row = e % T::ROWS; fi = e / T::ROWS; }
       // staged index of cell m is (m - seg0) + 3 = fi + 2
       int b = fi + 2;
-      if constexpr (CHAR) {
-        // characteristic fields of the stencil at the Roe average of cells m and m+1 (only
-        // the faces -1/2 .. n-1/2 are used)
-        int I[3];
-        bool ok = cell_of(row, fi - 1, I) && I[A] <= p.n[A] - 1;
-        if (ok) {
-          long long sl = pad_index(p, I[0], I[1], I[2]);
-          I[A] += 1;
-          long long sr = pad_index(p, I[0], I[1], I[2]);
-          double Ql[NV], Qr[NV];
+      // characteristic fields of the stencil at the Roe average of cells m and m+1 (only
+      // the faces -1/2 .. n-1/2 are used)
+      int I[3];
+      bool ok = cell_of(row, fi - 1, I) && I[A] <= p.n[A] - 1;
+      if (ok) {
+        long long sl = pad_index(p, I[0], I[1], I[2]);
+        I[A] += 1;
+        long long sr = pad_index(p, I[0], I[1], I[2]);
+        double Ql[NV], Qr[NV];
 #pragma unroll
-          for (int c = 0; c < NV; c++) {
-            Ql[c] = p.Qp[c * p.NP + sl];
-            Qr[c] = p.Qp[c * p.NP + sr];
-          }
-          double R[NV][NV], Lv[NV][NV];
-          roe_eigen<DIM, A>(p, Ql, Qr, R, Lv);
-          double hk[NV];
+        for (int c = 0; c < NV; c++) {
+          Ql[c] = p.Qp[c * p.NP + sl];
+          Qr[c] = p.Qp[c * p.NP + sr];
+        }
+        double R[NV][NV], Lv[NV][NV];
+        roe_eigen<DIM, A>(p, Ql, Qr, R, Lv);
+        double hk[NV];
 #pragma unroll
-          for (int k = 0; k < NV; k++) {
-            double vp[5], vm[5];
+        for (int k = 0; k < NV; k++) {
+          double vp[5], vm[5];
 #pragma unroll
-            for (int r = 0; r < 5; r++) {
-              double sp = 0.0, sn = 0.0;
+          for (int r = 0; r < 5; r++) {
+            double sp = 0.0, sn = 0.0;
 #pragma unroll
-              for (int c = 0; c < NV; c++) {
-                const double *fp = sfp + (c * T::ROWS + row) * T::LEN;
-                const double *fm = sfm + (c * T::ROWS + row) * T::LEN;
-                sp = sp + Lv[k][c] * fp[b - 2 + r];
-                sn = sn + Lv[k][c] * fm[b + 3 - r];
-              }
-              vp[r] = sp;
-              vm[r] = sn;
+            for (int c = 0; c < NV; c++) {
+              const double *fp = sfp + (c * T::ROWS + row) * T::LEN;
+              const double *fm = sfm + (c * T::ROWS + row) * T::LEN;
+              sp = sp + Lv[k][c] * fp[b - 2 + r];
+              sn = sn + Lv[k][c] * fm[b + 3 - r];
             }
-            hk[k] = recon<SCHEME>(p, vp[0], vp[1], vp[2], vp[3], vp[4]) +
-                    recon<SCHEME>(p, vm[0], vm[1], vm[2], vm[3], vm[4]);
+            vp[r] = sp;
+            vm[r] = sn;
           }
+          hk[k] = recon<SCHEME>(p, vp[0], vp[1], vp[2], vp[3], vp[4]) +
+                  recon<SCHEME>(p, vm[0], vm[1], vm[2], vm[3], vm[4]);
+        }
 #pragma unroll
-          for (int c = 0; c < NV; c++) {
-            double acc = 0.0;
+        for (int c = 0; c < NV; c++) {
+          double acc = 0.0;
 #pragma unroll
-            for (int k = 0; k < NV; k++) acc = acc + R[c][k] * hk[k];
-            Fh[ps][c] = acc;
-          }
-        } else {
-#pragma unroll
-          for (int c = 0; c < NV; c++) Fh[ps][c] = 0.0;
+          for (int k = 0; k < NV; k++) acc = acc + R[c][k] * hk[k];
+          Fh[ps][c] = acc;
         }
       } else {
 #pragma unroll
-        for (int c = 0; c < NV; c++) {
-          const double *fp = sfp + (c * T::ROWS + row) * T::LEN;
-          const double *fm = sfm + (c * T::ROWS + row) * T::LEN;
-          const double h = recon<SCHEME>(p, fp[b - 2], fp[b - 1], fp[b], fp[b + 1], fp[b + 2]) +
-                           recon<SCHEME>(p, fm[b + 3], fm[b + 2], fm[b + 1], fm[b], fm[b - 1]);
-          Fh[ps][c] = FOLD ? 0.5 * h : h;
-        }
+        for (int c = 0; c < NV; c++) Fh[ps][c] = 0.0;
       }
     }
   }
@@ -605,6 +760,151 @@ __global__ void __launch_bounds__(THREADS) k_conv(Plan p, int first) {
       double prev = first ? 0.0 : p.L[c * p.N + o];
       p.L[c * p.N + o] = prev - d;
     }
+  }
+}
+
+
+// Component-wise: a tile is 32 lines (y for A = 0, consecutive x otherwise) by up to 8 K faces of
+// one component; a warp takes the 32 lines of K consecutive faces.  The kernel is bound by the
+// FP64 pipe (1.7 lanes per clock and SM, so a warp instruction costs its SM quarter ~75 cycles):
+// what counts is FP64 operations, and that every SM quarter has several warps to issue them from.
+// Hence K faces per thread, whose differences are shared (faces_of_line), a block per component
+// (the split fluxes of one take 27 KB; a small grid has five times the blocks), segments of equal
+// length instead of a short last one, idle lanes only in whole warps, and a K chosen by the
+// launcher (conv_faces): 4 on large grids, less where tiles of 31 cells would leave SMs idle.
+// Against one face per thread on tiles of 63 (x) or 15 (y, z) cells with all components staged:
+// TENO5 at 256^3 x 8.06 -> 3.53 ms, y and z 5.92 -> 3.47 ms (FP64 operations per cell of a pass,
+// counted by ncu at 192^3 with K = 2: 121, before ~300 in x); WENO5-JS at 256^2 x 138 -> 70 us,
+// y 92 -> 70 us; strict TENO5 at 61 x 53 x 47 x 620 -> 242 us, y and z 961 -> 220 us.
+template <int A, int K>
+struct LineTile {
+  static constexpr int R = 32;                      // lines
+  static constexpr int FACES = (THREADS / 32) * K;  // faces per line
+  static constexpr int LEN = FACES + 5;             // staged cells per line (odd)
+  static constexpr int SL = A == 0 ? 1 : R, SR = A == 0 ? LEN : 1;      // staged strides
+  static constexpr int HL = A == 0 ? 1 : R, HR = A == 0 ? FACES + 1 : 1;  // face strides
+  static constexpr size_t BYTES = sizeof(double) * (2 * LEN * R + (FACES + 1) * R);
+};
+
+template <int DIM, int A, int SCHEME, int K>
+__global__ void __launch_bounds__(THREADS, 3) k_conv(Plan p, int first, int nseg) {
+  constexpr int NV = DIM + 2;
+  using T = LineTile<A, K>;
+  // TENO5's weights depend on ratios of indicators only (its floors aside), so its fast form
+  // reconstructs F +- alpha q and halves in the difference (a power of two: the same bits);
+  // WENO5-JS's eps = 1e-6 is not scale-free
+  constexpr bool FOLD = !STRICT && SCHEME == IBFSA_TENO5;
+  extern __shared__ double sm[];
+  double *sfp = sm;                   // f+ of the staged cells
+  double *sfm = sm + T::LEN * T::R;   // f-
+  double *sh = sfm + T::LEN * T::R;   // face fluxes
+  const double alpha = load_alpha(p, A);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int LN = A == 0 ? 1 : 0;  // direction of the tile's lines
+
+  const int c = blockIdx.x % NV;                    // component
+  const int segl = (p.n[A] + nseg - 1) / nseg;
+  const int seg0 = (blockIdx.x / NV % nseg) * segl;  // first cell along A
+  const int line0 = blockIdx.x / (NV * nseg) * T::R;
+  const int other = blockIdx.y;
+  const int ncell = min(segl, p.n[A] - seg0);
+  if (ncell <= 0) return;
+  const int nface = ncell + 1, nst = ncell + 6, nrow = min(T::R, p.n[LN] - line0);
+  int I[3] = {0, 0, 0};
+  I[A] = seg0;
+  I[LN] = line0;
+  if (DIM > 2) I[3 - A - LN] = other;
+  const long long stp[3] = {1, p.P[0], (long long)p.P[0] * p.P[1]};
+  const long long sti[3] = {1, p.n[0], (long long)p.n[0] * p.n[1]};
+  const double *Qb = p.Qp + pad_index(p, I[0], I[1], I[2]) - 3 * stp[A];
+  const double *Wb = p.Wp + pad_index(p, I[0], I[1], I[2]) - 3 * stp[A];
+  double *Lb = p.L + int_index(p, I[0], I[1], I[2]);
+
+  // the slots a warp's last faces read beyond the staged cells hold zeros
+  for (int l = nst - 1 + warp; l < T::LEN; l += THREADS / 32) {
+    sfm[lane * T::SR + l * T::SL] = 0.0;
+    if (l >= nst) sfp[lane * T::SR + l * T::SL] = 0.0;
+  }
+  // 1. split fluxes f+- = (F_A(Q) +- alpha Q)/2 of the staged cells, consecutive threads along x
+  constexpr int NS = (T::LEN * T::R + THREADS - 1) / THREADS;
+#pragma unroll
+  for (int i = 0; i < NS; i++) {
+    const int e = threadIdx.x + i * THREADS;
+    const int l = A == 0 ? e % nst : e / T::R, row = A == 0 ? e / nst : e % T::R;
+    if (l >= nst || row >= nrow) continue;
+    const int go = (int)(row * stp[LN] + l * stp[A]);
+    const double q = Qb[c * p.NP + go];
+    double F;
+    if (c == 0) {
+      F = Qb[(1 + A) * p.NP + go];
+    } else {
+      const double ua = Wb[A * p.NP + go], pr = Wb[DIM * p.NP + go];
+      if (c == NV - 1) {
+        F = (q + pr) * ua;
+      } else {
+        F = q * ua;
+        if (c - 1 == A) F += pr;
+      }
+    }
+    // f+ of staged cell l at l, f- at l - 1 (that of cell 0, which no face reads, lands on a
+    // slot that no face reads: the last one of the line before, or of f+)
+    const int so = row * T::SR + l * T::SL;
+    sfp[so] = FOLD ? fma(alpha, q, F) : 0.5 * (F + alpha * q);
+    sfm[so - T::SL] = FOLD ? fma(-alpha, q, F) : 0.5 * (F - alpha * q);
+  }
+  __syncthreads();
+  // 2. faces m+1/2, m = seg0 - 1 + fi: f+ of staged cells fi .. fi+4, f- of fi+1 .. fi+5
+  const int fi0 = warp * K;  // this warp's first face
+  if (fi0 < nface) {
+    const int at = min(lane, nrow - 1) * T::SR + fi0 * T::SL;
+    double f[K + 4], h[K], g[K];
+#pragma unroll
+    for (int j = 0; j < K + 4; j++) f[j] = sfp[at + j * T::SL];
+    unsigned fail = faces_of_line<SCHEME, false, K>(p, f, h);
+#pragma unroll
+    for (int j = 0; j < K + 4; j++) f[j] = sfm[at + j * T::SL];
+    fail |= faces_of_line<SCHEME, true, K>(p, f, g) << K;
+    if constexpr (SCHEME == IBFSA_TENO5) {
+      const unsigned some = (1u << min(K, nface - fi0)) - 1;  // slots that hold a face
+      fail &= some | some << K;
+      // full TENO5 where the sufficient test failed: each lane walks its own failed stencils
+      // (re-read from shared memory), one copy of the code
+#pragma unroll 1
+      while (fail) {
+        const int j = __ffs(fail) - 1;
+        fail &= fail - 1;
+        const double *v = j < K ? sfp + at + j * T::SL : sfm + at + (j - K + 4) * T::SL;
+        const int st = j < K ? T::SL : -T::SL;
+        const double t = teno5(p, v[0], v[st], v[2 * st], v[3 * st], v[4 * st]);
+#pragma unroll
+        for (int i = 0; i < K; i++) {
+          if (j == i) h[i] = t;
+          if (j == K + i) g[i] = t;
+        }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < K; j++) sh[lane * T::HR + (fi0 + j) * T::HL] = h[j] + g[j];
+  }
+  __syncthreads();
+  // 3. L = L - (Fhat_{m+1/2} - Fhat_{m-1/2}) / (dx/dxi); the boundary cell of a characteristic
+  // face takes its normal term from k_char_face instead.  A = 0: a warp walks the rows.
+  constexpr int NW = THREADS / 32;
+#pragma unroll
+  for (int i = 0; i < (A == 0 ? T::R / NW : (T::FACES + NW - 1) / NW); i++) {
+    const int row = A == 0 ? warp + i * NW : lane, l = A == 0 ? lane : warp + i * NW;
+    if (l >= ncell || row >= nrow) continue;
+    const double *hh = sh + row * T::HR + l * T::HL;
+    const double dh = hh[T::HL] - hh[0];
+    const int ia = seg0 + l;
+    constexpr double half = FOLD ? 0.5 : 1.0;
+    const bool str = p.mm[A] != nullptr;
+    const double inv = half * (str ? p.minv[A][ia + NG] : p.inv_h[A]);
+    double *Lc = Lb + c * p.N + row * sti[LN] + l * sti[A];
+    const double prev = first ? 0.0 : *Lc;
+    if (char_cell(p, A, ia)) *Lc = prev;
+    else if (STRICT) *Lc = prev - divide(dh, str ? p.mm[A][ia + NG] : p.h[A], inv);
+    else *Lc = fma(-dh, inv, prev);
   }
 }
 
@@ -691,6 +991,12 @@ __device__ __forceinline__ double d4(double fm2, double fm1, double fp1, double 
   return divide(8.0 * (fp1 - fm1) - (fp2 - fm2), h12, inv_h12);
 }
 
+// 12 dx/dxi at node i of direction a and its reciprocal, rounded as 12 h is on a uniform one
+__device__ __forceinline__ double metric12(const Plan &p, int a, int i, double *inv) {
+  *inv = p.mm[a] ? p.minv12[a][i + NG] : p.inv_h12[a];
+  return STRICT && p.mm[a] ? 12.0 * p.mm[a][i + NG] : p.h12[a];
+}
+
 template <int DIM>
 __global__ void __launch_bounds__(THREADS) k_visc_flux(Plan p) {
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -709,12 +1015,9 @@ __global__ void __launch_bounds__(THREADS) k_visc_flux(Plan p) {
 #pragma unroll
     for (int dj = 0; dj < DIM; dj++) {
       long long st = stride[dj];
-      if (p.mm[dj]) {  // 12 dx/dxi at this node, rounded as 12 h is on a uniform direction
-        int at = I[dj] + NG;
-        g[ci][dj] = d4(u[-2 * st], u[-st], u[st], u[2 * st], 12.0 * p.mm[dj][at], p.minv12[dj][at]);
-      } else {
-        g[ci][dj] = d4(u[-2 * st], u[-st], u[st], u[2 * st], p.h12[dj], p.inv_h12[dj]);
-      }
+      double inv;
+      const double h12 = metric12(p, dj, I[dj], &inv);
+      g[ci][dj] = d4(u[-2 * st], u[-st], u[st], u[2 * st], h12, inv);
     }
   }
   double div = 0.0;
@@ -751,12 +1054,9 @@ __global__ void __launch_bounds__(THREADS) k_visc_div(Plan p) {
     for (int a = 0; a < DIM; a++) {
       const double *F = p.V + (long long)(a * (DIM + 1) + fc) * p.NB + b;
       long long st = stride[a];
-      if (p.mm[a]) {
-        int at = (a == 0 ? i : a == 1 ? j : k) + NG;
-        sum += d4(F[-2 * st], F[-st], F[st], F[2 * st], 12.0 * p.mm[a][at], p.minv12[a][at]);
-      } else {
-        sum += d4(F[-2 * st], F[-st], F[st], F[2 * st], p.h12[a], p.inv_h12[a]);
-      }
+      double inv;
+      const double h12 = metric12(p, a, a == 0 ? i : a == 1 ? j : k, &inv);
+      sum += d4(F[-2 * st], F[-st], F[st], F[2 * st], h12, inv);
     }
     long long o = (long long)(fc + 1) * p.N + t;
     p.L[o] = p.L[o] + divide(sum, p.Re, p.inv_Re);
@@ -1013,14 +1313,11 @@ inline unsigned blocks_for(long long n, int threads) {
 }
 
 template <int DIM, int A, int SCHEME>
-cudaError_t launch_conv(const Plan &p, int first, cudaStream_t st) {
+cudaError_t launch_conv_char(const Plan &p, int first, cudaStream_t st) {
   using T = ConvTile<A>;
   constexpr size_t smem = conv_smem_bytes<DIM, A>();
-  cudaError_t e = p.charwise
-                      ? cudaFuncSetAttribute(k_conv<DIM, A, SCHEME, true>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                      : cudaFuncSetAttribute(k_conv<DIM, A, SCHEME, false>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(k_conv_char<DIM, A, SCHEME>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   dim3 grid;
   if (A == 0) {
@@ -1030,9 +1327,52 @@ cudaError_t launch_conv(const Plan &p, int first, cudaStream_t st) {
     int nx = (p.n[0] + T::ROWS - 1) / T::ROWS;
     grid = dim3(nseg * nx, A == 1 ? p.n[2] : p.n[1]);
   }
-  if (p.charwise) k_conv<DIM, A, SCHEME, true><<<grid, THREADS, smem, st>>>(p, first);
-  else k_conv<DIM, A, SCHEME, false><<<grid, THREADS, smem, st>>>(p, first);
+  k_conv_char<DIM, A, SCHEME><<<grid, THREADS, smem, st>>>(p, first);
   return cudaGetLastError();
+}
+
+// Faces per thread of k_conv: the K whose tiles (rowtiles: lines / 32 x components) give the
+// smallest (tiles of the busiest SM) x (FP64 operations of a tile), the tiles of a line being as
+// equal as they can be.  A face costs ~2 (4 + (K + 3)/K) + 1 operations, a staged cell ~3.
+// Measured, TENO5: 256^3, a y pass 3.47 / 3.82 / 4.91 ms with K = 4 / 2 / 1; WENO5-JS at 256^2,
+// where 31-cell tiles give 1.9 blocks per SM, 70 / 73 / 80 us; TENO5 at 383 x 257, x pass 59 / 50
+// / 54 us.
+inline int conv_faces(long long rowtiles, int n, int *nseg) {
+  int best = 4;
+  double cost = -1.0;
+  for (int K = 4; K >= 1; K /= 2) {
+    const int most = 8 * K - 1, ns = (n + most - 1) / most, seg = (n + ns - 1) / ns;
+    const double tile = (seg + 1) * (9.0 + 2.0 * (K + 3) / K) + 3.0 * (seg + 6) + 2.0 * seg;
+    const double c = (double)((rowtiles * ns + 151) / 152) * tile;
+    if (cost < 0.0 || c < cost) {
+      cost = c;
+      best = K;
+      *nseg = ns;
+    }
+  }
+  return best;
+}
+
+template <int DIM, int A, int SCHEME, int K>
+cudaError_t launch_conv_k(const Plan &p, int first, int nseg, long long tiles, cudaStream_t st) {
+  constexpr size_t smem = LineTile<A, K>::BYTES;
+  static_assert(smem <= 48 * 1024, "within the default dynamic shared memory");
+  static_assert(LineTile<A, K>::FACES <= 32, "the update walks a line of cells with one warp");
+  dim3 grid((unsigned)((DIM + 2) * tiles * nseg), A == 2 ? p.n[1] : p.n[2]);
+  k_conv<DIM, A, SCHEME, K><<<grid, THREADS, smem, st>>>(p, first, nseg);
+  return cudaGetLastError();
+}
+
+template <int DIM, int A, int SCHEME>
+cudaError_t launch_conv(const Plan &p, int first, cudaStream_t st) {
+  if (p.charwise) return launch_conv_char<DIM, A, SCHEME>(p, first, st);
+  const long long tiles = (p.n[A == 0 ? 1 : 0] + 31) / 32;
+  int nseg = 1;
+  switch (conv_faces((DIM + 2) * tiles * (A == 2 ? p.n[1] : p.n[2]), p.n[A], &nseg)) {
+    case 4: return launch_conv_k<DIM, A, SCHEME, 4>(p, first, nseg, tiles, st);
+    case 2: return launch_conv_k<DIM, A, SCHEME, 2>(p, first, nseg, tiles, st);
+    default: return launch_conv_k<DIM, A, SCHEME, 1>(p, first, nseg, tiles, st);
+  }
 }
 
 template <int DIM, int SCHEME>
