@@ -221,51 +221,86 @@ __device__ __forceinline__ float teno5_fast(const Plan &tw, float a, float b, fl
 // make_float2(v, v)
 __device__ __forceinline__ float2 f2(float v) { return make_float2(v, v); }
 
-// TENO5 at one face for both split fluxes on packed FP32x2 arithmetic, with a warp-uniform slow
-// path: every lane of the warp must call it.  The input is the interleaved face stencil
-// z_k = (f+ at staged cell i+k, f- at staged cell i+k+1), k = 0..4, of the face between staged
-// cells i+2 and i+3: the .x lanes are the f+ stencil upwind to downwind, the .y lanes the f-
-// stencil downwind to upwind, so one 8-byte load per k fetches both sides.  With the f- stencil
-// reversed, the packed indicator of z0 z1 z2 is (beta_0+, beta_2-) and that of z2 z3 z4 is
-// (beta_2+, beta_0-) (the second differences and the squared one-sided differences are
+// Two adjacent faces, both split fluxes each, on packed FP32x2 arithmetic.  The input is the
+// interleaved face stencils z_k = (f+ at staged cell i+k, f- at staged cell i+k+1), k = 0..5, of
+// the faces after staged cells i+2 and i+3: the .x lanes are the f+ stencils upwind to downwind,
+// the .y lanes the f- stencils downwind to upwind, so one load per k fetches both sides.  First
+// differences, second differences and their squares are taken once for both faces (each face by
+// itself: 26 packed operations, the pair: 41; the passes are bound by instruction issue).  At 512^3
+// with TENO5 x 2.27 -> 1.97 ms, y and z 2.36 -> 2.22 ms; WENO5-JS at 2048^2, before one side and
+// component at a time without packing, x 95 -> 67 us, y 101 -> 70 us.  With the f- stencil reversed, the packed indicator
+// of z0 z1 z2 is (beta_0+, beta_2-) and that of z2 z3 z4 is (beta_2+, beta_0-) (the squares are
 // symmetric under the reversal), so tau5 and the all-kept test are those of each side; the
-// linear combination takes per-lane coefficient pairs.  The all-kept test is scale-invariant, so
-// the indicators are taken times 4, (13/3) t^2 + u^2 (one multiplication fewer each), with the
-// floor 4e-30.  The linear (all-kept) result is computed without branches; only when some lane
-// of the warp has a side that cuts a stencil does the whole warp enter the full TENO5 (a uniform
-// branch, no divergence to reconverge).
-__device__ __forceinline__ float teno5_pz_warp(const Plan &tw, float2 z0, float2 z1, float2 z2,
-                                               float2 z3, float2 z4) {
-  float2 t0 = __fadd2_rn(__ffma2_rn(f2(-2.f), z1, z0), z2);
-  float2 t1 = __fadd2_rn(__ffma2_rn(f2(-2.f), z2, z1), z3);
-  float2 t2 = __fadd2_rn(__ffma2_rn(f2(-2.f), z3, z2), z4);
-  float2 u0 = __ffma2_rn(f2(3.f), z2, __ffma2_rn(f2(-4.f), z1, z0));
-  float2 u1 = __ffma2_rn(f2(-1.f), z3, z1);
-  float2 u2 = __ffma2_rn(f2(3.f), z2, __ffma2_rn(f2(-4.f), z3, z4));
-  const float2 k13 = f2(13.f / 3.f);
-  float2 b0 = __ffma2_rn(__fmul2_rn(k13, t0), t0, __fmul2_rn(u0, u0));
-  float2 b1 = __ffma2_rn(__fmul2_rn(k13, t1), t1, __fmul2_rn(u1, u1));
-  float2 b2 = __ffma2_rn(__fmul2_rn(k13, t2), t2, __fmul2_rn(u2, u2));
-  float2 tau = __ffma2_rn(f2(-1.f), b2, b0);
-  const bool kx = fabsf(tau.x) <= fmaf(4.f, fminf(b0.x, fminf(b1.x, b2.x)), 1.6e-29f);
-  const bool ky = fabsf(tau.y) <= fmaf(4.f, fminf(b0.y, fminf(b1.y, b2.y)), 1.6e-29f);
-  float2 lin = __fmul2_rn(make_float2(2.f / 60.f, -3.f / 60.f), z0);
-  lin = __ffma2_rn(make_float2(-13.f / 60.f, 27.f / 60.f), z1, lin);
-  lin = __ffma2_rn(f2(47.f / 60.f), z2, lin);
-  lin = __ffma2_rn(make_float2(27.f / 60.f, -13.f / 60.f), z3, lin);
-  lin = __ffma2_rn(make_float2(-3.f / 60.f, 2.f / 60.f), z4, lin);
-  float h = lin.x + lin.y;
-  if (__any_sync(0xffffffffu, !(kx && ky))) {
-    float hx = kx ? lin.x : teno5(tw, z0.x, z1.x, z2.x, z3.x, z4.x);
-    float hy = ky ? lin.y : teno5(tw, z4.y, z3.y, z2.y, z1.y, z0.y);
-    h = hx + hy;
+// linear combination takes per-lane coefficient pairs.
+//
+// TENO5: the all-kept test is scale-invariant, so the indicators are taken times 4, (13/3) t^2 +
+// u^2, with the floor 4e-30.  The linear (all-kept) result is computed without branches; only
+// when some lane of the warp has a side that cuts a stencil does the whole warp enter the full
+// TENO5 (a uniform branch, no divergence to reconverge): every lane of the warp must call it, and
+// v0, v1 say which of its faces exist.
+// WENO5-JS: weights d_k / (eps + beta_k)^2 over their common denominator, the reconstruction as
+// the middle value plus a weighted mean of the candidates' differences from it.
+template <int SCHEME>
+__device__ __forceinline__ void faces_pz2(const Plan &tw, const float2 (&z)[6], bool v0, bool v1,
+                                          float (&h)[2]) {
+  float2 d[5], kt[4];
+#pragma unroll
+  for (int j = 0; j < 5; j++) d[j] = __ffma2_rn(f2(-1.f), z[j], z[j + 1]);
+#pragma unroll
+  for (int j = 0; j < 4; j++) {
+    const float2 t = __ffma2_rn(f2(-1.f), d[j], d[j + 1]);
+    // WENO5-JS: the indicators themselves (times 1) plus eps
+    if constexpr (SCHEME == IBFSA_TENO5) kt[j] = __fmul2_rn(__fmul2_rn(f2(13.f / 3.f), t), t);
+    else kt[j] = __ffma2_rn(__fmul2_rn(f2(13.f / 12.f), t), t, f2(1e-6f));
   }
-  return h;
+#pragma unroll
+  for (int j = 0; j < 2; j++) {
+    const float2 u0 = __ffma2_rn(f2(-3.f), d[j + 1], d[j]);
+    const float2 u1 = __fadd2_rn(d[j + 1], d[j + 2]);
+    const float2 u2 = __ffma2_rn(f2(-3.f), d[j + 2], d[j + 3]);
+    if constexpr (SCHEME == IBFSA_TENO5) {
+      const float2 b0 = __ffma2_rn(u0, u0, kt[j]), b1 = __ffma2_rn(u1, u1, kt[j + 1]);
+      const float2 b2 = __ffma2_rn(u2, u2, kt[j + 2]);
+      const float2 tau = __ffma2_rn(f2(-1.f), b2, b0);
+      const bool kx = fabsf(tau.x) <= fmaf(4.f, fminf(b0.x, fminf(b1.x, b2.x)), 1.6e-29f);
+      const bool ky = fabsf(tau.y) <= fmaf(4.f, fminf(b0.y, fminf(b1.y, b2.y)), 1.6e-29f);
+      float2 lin = __fmul2_rn(make_float2(2.f / 60.f, -3.f / 60.f), z[j]);
+      lin = __ffma2_rn(make_float2(-13.f / 60.f, 27.f / 60.f), z[j + 1], lin);
+      lin = __ffma2_rn(f2(47.f / 60.f), z[j + 2], lin);
+      lin = __ffma2_rn(make_float2(27.f / 60.f, -13.f / 60.f), z[j + 3], lin);
+      lin = __ffma2_rn(make_float2(-3.f / 60.f, 2.f / 60.f), z[j + 4], lin);
+      h[j] = lin.x + lin.y;
+      if (__any_sync(0xffffffffu, (j ? v1 : v0) && !(kx && ky))) {
+        const float hx = kx ? lin.x : teno5(tw, z[j].x, z[j + 1].x, z[j + 2].x, z[j + 3].x, z[j + 4].x);
+        const float hy = ky ? lin.y : teno5(tw, z[j + 4].y, z[j + 3].y, z[j + 2].y, z[j + 1].y, z[j].y);
+        h[j] = hx + hy;
+      }
+    } else {
+      const float2 q = f2(0.25f);
+      float2 b0 = __ffma2_rn(__fmul2_rn(q, u0), u0, kt[j]);
+      float2 b1 = __ffma2_rn(__fmul2_rn(q, u1), u1, kt[j + 1]);
+      float2 b2 = __ffma2_rn(__fmul2_rn(q, u2), u2, kt[j + 2]);
+      b0 = __fmul2_rn(b0, b0);
+      b1 = __fmul2_rn(b1, b1);
+      b2 = __fmul2_rn(b2, b2);
+      const float2 p0 = __fmul2_rn(b1, b2), p1 = __fmul2_rn(b0, b2), p2 = __fmul2_rn(b0, b1);
+      const float2 n0 = __ffma2_rn(make_float2(5.f / 60.f, -12.f / 60.f), d[j + 1],
+                                   __fmul2_rn(make_float2(-2.f / 60.f, 3.f / 60.f), d[j]));
+      const float2 n1 = __ffma2_rn(make_float2(0.1f, -0.2f), d[j + 1],
+                                   __fmul2_rn(make_float2(0.2f, -0.1f), d[j + 2]));
+      const float2 n2 = __ffma2_rn(make_float2(12.f / 60.f, -5.f / 60.f), d[j + 2],
+                                   __fmul2_rn(make_float2(-3.f / 60.f, 2.f / 60.f), d[j + 3]));
+      const float2 num = __ffma2_rn(p2, n2, __ffma2_rn(p1, n1, __fmul2_rn(p0, n0)));
+      const float2 den = __ffma2_rn(make_float2(0.3f, 0.1f), p2,
+                                    __ffma2_rn(f2(0.6f), p1, __fmul2_rn(make_float2(0.1f, 0.3f), p0)));
+      h[j] = (z[j + 2].x + __fdividef(num.x, den.x)) + (z[j + 2].y + __fdividef(num.y, den.y));
+    }
+  }
 }
 
-// teno5_pz_warp per side: returns (h+, h-) and whether each side keeps all three stencils (by
-// the all-kept test or, where that fails, by the full cut-off).  Every lane of the warp must call
-// it.
+// TENO5 at one face of the interleaved stencils (faces_pz2): (h+, h-) and whether each side keeps
+// all three stencils (by the all-kept test or, where that fails, by the full cut-off).  Every lane
+// of the warp must call it.
 __device__ __forceinline__ float2 teno5_pz_sides(const Plan &tw, float2 z0, float2 z1, float2 z2,
                                                  float2 z3, float2 z4, bool &kx, bool &ky) {
   float2 t0 = __fadd2_rn(__ffma2_rn(f2(-2.f), z1, z0), z2);
@@ -485,7 +520,7 @@ struct Tile {
   // faces per thread either way
   static constexpr int ROWS = A == 0 ? 8 : 32;
   static constexpr int SEG = A == 0 ? 63 : 15;
-  static constexpr int LEN = SEG + 6;
+  static constexpr int LEN = SEG + 6 + (A == 0 ? 1 : 0);  // x: even, so that rows keep 16 bytes
   static constexpr int FACES = SEG + 1;
 };
 
@@ -594,11 +629,12 @@ __device__ __forceinline__ void roe_eigen32(const Free &fs, const float wl[DIM +
   }
 }
 
-// eight blocks per SM (32 registers) for the fixed schemes, four (64 registers) for the
-// learned form's warp-wide network tiles, one for the characteristic-wise option (its two
-// eigen-systems per face take registers).  The x pass gives each warp one row of the tile.
+// Six blocks per SM (42 registers) for the fixed schemes' pairs of faces (x pass at 512^3 1.97 ms;
+// with 4 / 5 / 8 blocks 2.07 / 2.00 / 2.13), four (64 registers) for the learned form's warp-wide
+// network tiles, one for the characteristic-wise option (its two eigen-systems per face take
+// registers).  The x pass gives each warp one row of the tile.
 template <int DIM, int A, int SCHEME, bool CHAR = false>
-__global__ void __launch_bounds__(THREADS, SCHEME == IBFSA_MLP_TENO5 ? 4 : (CHAR ? 1 : 8))
+__global__ void __launch_bounds__(THREADS, SCHEME == IBFSA_MLP_TENO5 ? 4 : (CHAR ? 1 : 6))
     k_conv32(Plan p, int first) {
   constexpr int NV = DIM + 2;
   using T = Tile<A>;
@@ -607,10 +643,11 @@ __global__ void __launch_bounds__(THREADS, SCHEME == IBFSA_MLP_TENO5 ? 4 : (CHAR
   // 32 lanes hit 32 different banks
   constexpr int FST = A == 0 ? T::FACES : T::FACES + 1;
   extern __shared__ float smf[];
-  // component-wise TENO5 and the learned weights stage the interleaved face stencils
-  // z_l = (f+ at l, f- at l+1), [NV][ROWS][LEN] float2 (teno5_pz_warp); the other schemes f+ and
-  // f- apart, [NV][ROWS][LEN]
-  constexpr bool ZL = (SCHEME == IBFSA_TENO5 || SCHEME == IBFSA_MLP_TENO5) && !CHAR;
+  // the component-wise forms stage the interleaved face stencils z_l = (f+ at l, f- at l+1),
+  // [NV][ROWS][LEN] float2; the characteristic-wise option f+ and f- apart, [NV][ROWS][LEN]
+  constexpr bool ZL = !CHAR;
+  // faces of a thread: one row's adjacent pair (component-wise), or THREADS apart
+  constexpr bool PAIR = !CHAR && SCHEME != IBFSA_MLP_TENO5;
   float *sfp = smf;
   float *sfm = smf + NV * T::ROWS * T::LEN;
   const float alpha = (float)__longlong_as_double((long long)p.alpha_bits[A]);
@@ -766,36 +803,34 @@ __global__ void __launch_bounds__(THREADS, SCHEME == IBFSA_MLP_TENO5 ? 4 : (CHAR
       }
     }
   } else {
+    // the thread's pair of adjacent faces fi, fi + 1 (face fi + 1/2 - 1 between staged cells fi + 2
+    // and fi + 3: z_fi .. z_fi+4).  Every lane of the warp takes part (the slow path is warp-
+    // uniform): lanes without a face evaluate a valid one and store nothing.
+    static_assert(MAXP == 2, "two faces per thread");
+    int row = A == 0 ? warp : lane, fi = 2 * (A == 0 ? lane : warp);
+    const bool v0 = row < nrow && fi < nface, v1 = row < nrow && fi + 1 < nface;
+    if (!v0) fi = 0;
+    if (row >= nrow) row = 0;
+    const float2 *zr = reinterpret_cast<const float2 *>(smf) + row * T::LEN + fi;
 #pragma unroll
-    for (int ps = 0; ps < MAXP; ps++) {
-      int e = threadIdx.x + ps * THREADS;
-      int row, fi;
-      if constexpr (A == 0) { row = e / T::FACES; fi = e % T::FACES; }
-      else { row = e % T::ROWS; fi = e / T::ROWS; }
-      if constexpr (SCHEME == IBFSA_TENO5) {
-        // every lane of the warp takes part (the slow path is warp-uniform): lanes without a
-        // face evaluate a valid one of their row (or row 0) and store nothing
-        const bool valid = e < T::ROWS * T::FACES && row < nrow && fi < nface;
-        if (!valid) {
-          fi = 0;
-          if (row >= nrow) row = 0;
-        }
-        // face fi + 1/2 - 1 between staged cells fi + 2 and fi + 3: z_fi .. z_fi+4
+    for (int c = 0; c < NV; c++) {
+      float2 z[6];
+      if constexpr (A == 0) {  // 16-byte loads: fi and the row pitch are even
+        const float4 *z4 = reinterpret_cast<const float4 *>(zr + c * T::ROWS * T::LEN);
 #pragma unroll
-        for (int c = 0; c < NV; c++) {
-          const float2 *z = reinterpret_cast<const float2 *>(smf) + (c * T::ROWS + row) * T::LEN + fi;
-          Fh[ps][c] = teno5_pz_warp(p, z[0], z[1], z[2], z[3], z[4]);
+        for (int j = 0; j < 3; j++) {
+          const float4 v = z4[j];
+          z[2 * j] = make_float2(v.x, v.y);
+          z[2 * j + 1] = make_float2(v.z, v.w);
         }
-      } else if (e < T::ROWS * T::FACES && row < nrow && fi < nface) {
-        int b = fi + 2;
+      } else {
 #pragma unroll
-        for (int c = 0; c < NV; c++) {
-          const float *fp = sfp + (c * T::ROWS + row) * T::LEN;
-          const float *fm = sfm + (c * T::ROWS + row) * T::LEN;
-          Fh[ps][c] = recon<SCHEME>(p, fp[b - 2], fp[b - 1], fp[b], fp[b + 1], fp[b + 2]) +
-                      recon<SCHEME>(p, fm[b + 3], fm[b + 2], fm[b + 1], fm[b], fm[b - 1]);
-        }
+        for (int j = 0; j < 6; j++) z[j] = zr[c * T::ROWS * T::LEN + j];
       }
+      float h[2];
+      faces_pz2<SCHEME>(p, z, v0, v1, h);
+      Fh[0][c] = h[0];
+      Fh[1][c] = h[1];
     }
   }
   __syncthreads();
@@ -804,7 +839,8 @@ __global__ void __launch_bounds__(THREADS, SCHEME == IBFSA_MLP_TENO5 ? 4 : (CHAR
   for (int ps = 0; ps < MAXP; ps++) {
     int e = threadIdx.x + ps * THREADS;
     int row, fi;
-    if constexpr (A == 0) { row = e / T::FACES; fi = e % T::FACES; }
+    if constexpr (PAIR) { row = A == 0 ? warp : lane; fi = 2 * (A == 0 ? lane : warp) + ps; }
+    else if constexpr (A == 0) { row = e / T::FACES; fi = e % T::FACES; }
     else { row = e % T::ROWS; fi = e / T::ROWS; }
     if (e < T::ROWS * T::FACES && row < nrow && fi < nface) {
 #pragma unroll
@@ -889,8 +925,8 @@ __global__ void __launch_bounds__(THREADS, SCHEME == IBFSA_MLP_TENO5 ? 4 : 5)
   using T = Tile<A>;
   constexpr int NV = TT::NV, R = TT::R, LEN = TT::LEN, SEG = TT::SEG;
   constexpr int FST = T::FACES + 1;
-  // TENO5 and the learned weights stage interleaved face stencils z_l = (f+ at l, f- at l+1)
-  constexpr bool ZL = SCHEME == IBFSA_TENO5 || SCHEME == IBFSA_MLP_TENO5;
+  // faces of a thread: an adjacent pair (fixed schemes), or NW apart (learned weights)
+  constexpr bool PAIR = SCHEME != IBFSA_MLP_TENO5;
   extern __shared__ __align__(128) float smf[];
   float *in = smf;                         // [NV + 2][LEN][R], then L' [NV][SEG][R]
   float *sfp = smf + TT::IN;               // [NV][LEN - 1][R]: f+ at staged cells 0..LEN-2
@@ -936,20 +972,12 @@ __global__ void __launch_bounds__(THREADS, SCHEME == IBFSA_MLP_TENO5 ? 4 : 5)
       for (int c = 0; c < NV; c++) q[c] = in[(c * LEN + l) * R + lane];
       split_cell<DIM, A>(fs, alpha, q, in[(NV * LEN + l) * R + lane],
                          in[((NV + 1) * LEN + l) * R + lane], fpv, fmv);
-      if constexpr (ZL) {
-        // interleaved face stencils z_l = (f+ at l, f- at l+1), [NV][LEN-1][R] float2
-        float2 *Z = reinterpret_cast<float2 *>(sfp);
+      // interleaved face stencils z_l = (f+ at l, f- at l+1), [NV][LEN-1][R] float2
+      float2 *Z = reinterpret_cast<float2 *>(sfp);
 #pragma unroll
-        for (int c = 0; c < NV; c++) {
-          if (l < LEN - 1) Z[(c * (LEN - 1) + l) * R + lane].x = fpv[c];
-          if (l > 0) Z[(c * (LEN - 1) + l - 1) * R + lane].y = fmv[c];
-        }
-      } else {
-#pragma unroll
-        for (int c = 0; c < NV; c++) {
-          if (l < LEN - 1) sfp[(c * (LEN - 1) + l) * R + lane] = fpv[c];
-          if (l > 0) sfm[(c * (LEN - 1) + l - 1) * R + lane] = fmv[c];
-        }
+      for (int c = 0; c < NV; c++) {
+        if (l < LEN - 1) Z[(c * (LEN - 1) + l) * R + lane].x = fpv[c];
+        if (l > 0) Z[(c * (LEN - 1) + l - 1) * R + lane].y = fmv[c];
       }
     }
   }
@@ -980,30 +1008,27 @@ __global__ void __launch_bounds__(THREADS, SCHEME == IBFSA_MLP_TENO5 ? 4 : 5)
       atomicAdd(&p.mlp_counts[1], (unsigned long long)seen);
     }
   } else {
-#pragma unroll
-  for (int ps = 0; ps < MAXP; ps++) {
-    const int fi = warp + ps * NW;
+    static_assert(MAXP == 2, "two faces per thread");
+    const int fi = 2 * warp;  // the same for the whole warp
     if (fi < nface) {
 #pragma unroll
       for (int c = 0; c < NV; c++) {
-        if constexpr (SCHEME == IBFSA_TENO5) {  // fi is the same for the whole warp
-          const float2 *z = reinterpret_cast<const float2 *>(sfp) + (c * (LEN - 1) + fi) * R + lane;
-          Fh[ps][c] = teno5_pz_warp(p, z[0], z[R], z[2 * R], z[3 * R], z[4 * R]);
-        } else {
-          const float *fp = sfp + (c * (LEN - 1) + fi) * R + lane;
-          const float *fm = sfm + (c * (LEN - 1) + fi) * R + lane;   // f- of staged cell fi+1
-          Fh[ps][c] = recon<SCHEME>(p, fp[0], fp[R], fp[2 * R], fp[3 * R], fp[4 * R]) +
-                      recon<SCHEME>(p, fm[4 * R], fm[3 * R], fm[2 * R], fm[R], fm[0]);
-        }
+        const float2 *zc = reinterpret_cast<const float2 *>(sfp) + (c * (LEN - 1) + fi) * R + lane;
+        float2 z[6];
+#pragma unroll
+        for (int j = 0; j < 6; j++) z[j] = zc[j * R];
+        float h[2];
+        faces_pz2<SCHEME>(p, z, row_ok, row_ok && fi + 1 < nface, h);
+        Fh[0][c] = h[0];
+        Fh[1][c] = h[1];
       }
     }
-  }
   }
   __syncthreads();
   float *sh = sfp;  // face fluxes [NV][R][FST]
 #pragma unroll
   for (int ps = 0; ps < MAXP; ps++) {
-    const int fi = warp + ps * NW;
+    const int fi = PAIR ? 2 * warp + ps : warp + ps * NW;
     if (fi < nface) {
 #pragma unroll
       for (int c = 0; c < NV; c++) sh[(c * R + lane) * FST + fi] = Fh[ps][c];
