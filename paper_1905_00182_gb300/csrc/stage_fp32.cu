@@ -170,10 +170,12 @@ __device__ __forceinline__ int teno_mask(const Cands &k) {
   return (g0 >= th ? 1 : 0) | (g1 >= th ? 2 : 0) | (g2 >= th ? 4 : 0);
 }
 
+// E: factor of the indicators' floor, for stencils scaled by its square root
+template <int E = 1>
 __device__ __forceinline__ float teno5(const Plan &tw, float a, float b, float c, float d,
                                        float e) {
   Cands k = candidates(a, b, c, d, e);
-  const float eps = 1e-30f, CT = 1e-5f;
+  const float eps = E * 1e-30f, CT = 1e-5f;
   float tau = fabsf(k.b0 - k.b2);
   float r0 = __fdividef(tau, k.b0 + eps);
   float r1 = __fdividef(tau, k.b1 + eps);
@@ -221,9 +223,9 @@ __device__ __forceinline__ float teno5_fast(const Plan &tw, float a, float b, fl
 // make_float2(v, v)
 __device__ __forceinline__ float2 f2(float v) { return make_float2(v, v); }
 
-// Two adjacent faces, both split fluxes each, on packed FP32x2 arithmetic.  The input is the
-// interleaved face stencils z_k = (f+ at staged cell i+k, f- at staged cell i+k+1), k = 0..5, of
-// the faces after staged cells i+2 and i+3: the .x lanes are the f+ stencils upwind to downwind,
+// K adjacent faces (2, or 1), both split fluxes each, on packed FP32x2 arithmetic.  The input is
+// the interleaved face stencils z_k = (f+ at staged cell i+k, f- at staged cell i+k+1), k = 0..K+3,
+// of the faces after staged cells i+2, i+3: the .x lanes are the f+ stencils upwind to downwind,
 // the .y lanes the f- stencils downwind to upwind, so one load per k fetches both sides.  First
 // differences, second differences and their squares are taken once for both faces (each face by
 // itself: 26 packed operations, the pair: 41; the passes are bound by instruction issue).  At 512^3
@@ -234,36 +236,36 @@ __device__ __forceinline__ float2 f2(float v) { return make_float2(v, v); }
 // linear combination takes per-lane coefficient pairs.
 //
 // TENO5: the all-kept test is scale-invariant, so the indicators are taken times 4, (13/3) t^2 +
-// u^2, with the floor 4e-30.  The linear (all-kept) result is computed without branches; only
+// u^2, of twice the split flux (STAGE_SCALE), with the floor 16e-30.  The linear (all-kept) result is computed without branches; only
 // when some lane of the warp has a side that cuts a stencil does the whole warp enter the full
 // TENO5 (a uniform branch, no divergence to reconverge): every lane of the warp must call it, and
 // v0, v1 say which of its faces exist.
 // WENO5-JS: weights d_k / (eps + beta_k)^2 over their common denominator, the reconstruction as
 // the middle value plus a weighted mean of the candidates' differences from it.
-template <int SCHEME>
-__device__ __forceinline__ void faces_pz2(const Plan &tw, const float2 (&z)[6], bool v0, bool v1,
-                                          float (&h)[2]) {
-  float2 d[5], kt[4];
+template <int SCHEME, int K>
+__device__ __forceinline__ void faces_pz(const Plan &tw, const float2 (&z)[K + 4], bool v0, bool v1,
+                                         float (&h)[K]) {
+  float2 d[K + 3], kt[K + 2];
 #pragma unroll
-  for (int j = 0; j < 5; j++) d[j] = __ffma2_rn(f2(-1.f), z[j], z[j + 1]);
+  for (int j = 0; j < K + 3; j++) d[j] = __ffma2_rn(f2(-1.f), z[j], z[j + 1]);
 #pragma unroll
-  for (int j = 0; j < 4; j++) {
+  for (int j = 0; j < K + 2; j++) {
     const float2 t = __ffma2_rn(f2(-1.f), d[j], d[j + 1]);
-    // WENO5-JS: the indicators themselves (times 1) plus eps
+    // WENO5-JS: eps with the indicator (four times that of half the split flux)
     if constexpr (SCHEME == IBFSA_TENO5) kt[j] = __fmul2_rn(__fmul2_rn(f2(13.f / 3.f), t), t);
-    else kt[j] = __ffma2_rn(__fmul2_rn(f2(13.f / 12.f), t), t, f2(1e-6f));
+    else kt[j] = __ffma2_rn(__fmul2_rn(f2(13.f / 3.f), t), t, f2(1e-6f));
   }
 #pragma unroll
-  for (int j = 0; j < 2; j++) {
+  for (int j = 0; j < K; j++) {
     const float2 u0 = __ffma2_rn(f2(-3.f), d[j + 1], d[j]);
     const float2 u1 = __fadd2_rn(d[j + 1], d[j + 2]);
     const float2 u2 = __ffma2_rn(f2(-3.f), d[j + 2], d[j + 3]);
+    float2 b0 = __ffma2_rn(u0, u0, kt[j]), b1 = __ffma2_rn(u1, u1, kt[j + 1]);
+    float2 b2 = __ffma2_rn(u2, u2, kt[j + 2]);
     if constexpr (SCHEME == IBFSA_TENO5) {
-      const float2 b0 = __ffma2_rn(u0, u0, kt[j]), b1 = __ffma2_rn(u1, u1, kt[j + 1]);
-      const float2 b2 = __ffma2_rn(u2, u2, kt[j + 2]);
       const float2 tau = __ffma2_rn(f2(-1.f), b2, b0);
-      const bool kx = fabsf(tau.x) <= fmaf(4.f, fminf(b0.x, fminf(b1.x, b2.x)), 1.6e-29f);
-      const bool ky = fabsf(tau.y) <= fmaf(4.f, fminf(b0.y, fminf(b1.y, b2.y)), 1.6e-29f);
+      const bool kx = fabsf(tau.x) <= fmaf(4.f, fminf(b0.x, fminf(b1.x, b2.x)), 6.4e-29f);
+      const bool ky = fabsf(tau.y) <= fmaf(4.f, fminf(b0.y, fminf(b1.y, b2.y)), 6.4e-29f);
       float2 lin = __fmul2_rn(make_float2(2.f / 60.f, -3.f / 60.f), z[j]);
       lin = __ffma2_rn(make_float2(-13.f / 60.f, 27.f / 60.f), z[j + 1], lin);
       lin = __ffma2_rn(f2(47.f / 60.f), z[j + 2], lin);
@@ -271,15 +273,11 @@ __device__ __forceinline__ void faces_pz2(const Plan &tw, const float2 (&z)[6], 
       lin = __ffma2_rn(make_float2(-3.f / 60.f, 2.f / 60.f), z[j + 4], lin);
       h[j] = lin.x + lin.y;
       if (__any_sync(0xffffffffu, (j ? v1 : v0) && !(kx && ky))) {
-        const float hx = kx ? lin.x : teno5(tw, z[j].x, z[j + 1].x, z[j + 2].x, z[j + 3].x, z[j + 4].x);
-        const float hy = ky ? lin.y : teno5(tw, z[j + 4].y, z[j + 3].y, z[j + 2].y, z[j + 1].y, z[j].y);
+        const float hx = kx ? lin.x : teno5<4>(tw, z[j].x, z[j + 1].x, z[j + 2].x, z[j + 3].x, z[j + 4].x);
+        const float hy = ky ? lin.y : teno5<4>(tw, z[j + 4].y, z[j + 3].y, z[j + 2].y, z[j + 1].y, z[j].y);
         h[j] = hx + hy;
       }
     } else {
-      const float2 q = f2(0.25f);
-      float2 b0 = __ffma2_rn(__fmul2_rn(q, u0), u0, kt[j]);
-      float2 b1 = __ffma2_rn(__fmul2_rn(q, u1), u1, kt[j + 1]);
-      float2 b2 = __ffma2_rn(__fmul2_rn(q, u2), u2, kt[j + 2]);
       b0 = __fmul2_rn(b0, b0);
       b1 = __fmul2_rn(b1, b1);
       b2 = __fmul2_rn(b2, b2);
@@ -298,7 +296,7 @@ __device__ __forceinline__ void faces_pz2(const Plan &tw, const float2 (&z)[6], 
   }
 }
 
-// TENO5 at one face of the interleaved stencils (faces_pz2): (h+, h-) and whether each side keeps
+// TENO5 at one face of the interleaved stencils (faces_pz): (h+, h-) and whether each side keeps
 // all three stencils (by the all-kept test or, where that fails, by the full cut-off).  Every lane
 // of the warp must call it.
 __device__ __forceinline__ float2 teno5_pz_sides(const Plan &tw, float2 z0, float2 z1, float2 z2,
@@ -520,7 +518,7 @@ struct Tile {
   // faces per thread either way
   static constexpr int ROWS = A == 0 ? 8 : 32;
   static constexpr int SEG = A == 0 ? 63 : 15;
-  static constexpr int LEN = SEG + 6 + (A == 0 ? 1 : 0);  // x: even, so that rows keep 16 bytes
+  static constexpr int LEN = SEG + 6;
   static constexpr int FACES = SEG + 1;
 };
 
@@ -529,9 +527,19 @@ constexpr size_t conv_smem() {
   return sizeof(float) * 2 * (DIM + 2) * Tile<A>::ROWS * Tile<A>::LEN;  // >= face-flux area
 }
 
-// split fluxes f+-' = (F' +- alpha q') / 2 along A of one staged cell, from q', u'_A and p';
-// F' is the perturbation-expanded flux (no O(1) free-stream terms cancel)
-template <int DIM, int A>
+// What the split fluxes f+-' = (F' +- alpha q') / 2 are staged as (a power of two: the same bits):
+// the fixed component-wise schemes stage F' +- alpha q' itself for TENO5, which depends on ratios of
+// indicators only (its floors take the square of the scale), and half of f+-' for WENO5-JS, whose
+// indicators (eps is not scale-free) come out times four; every other form (-1) stages f+-'.
+template <int SCHEME>
+constexpr float STAGE_SCALE = SCHEME < 0 ? 0.5f : SCHEME == IBFSA_TENO5 ? 1.f : 0.25f;
+// and what takes a flux difference back
+template <int SCHEME>
+constexpr float FLUX_SCALE = 0.5f / STAGE_SCALE<SCHEME>;
+
+// split fluxes along A of one staged cell, from q', u'_A and p'; F' is the perturbation-expanded
+// flux (no O(1) free-stream terms cancel)
+template <int DIM, int A, int SCHEME = -1>
 __device__ __forceinline__ void split_cell(const Free &fs, float alpha, const float q[DIM + 2],
                                            float up, float pp, float fpv[DIM + 2],
                                            float fmv[DIM + 2]) {
@@ -547,8 +555,8 @@ __device__ __forceinline__ void split_cell(const Free &fs, float alpha, const fl
       if (c - 1 == A) F += pp;
     }
     const float aq = alpha * q[c];
-    fpv[c] = 0.5f * (F + aq);
-    fmv[c] = 0.5f * (F - aq);
+    fpv[c] = STAGE_SCALE<SCHEME> * (F + aq);
+    fmv[c] = STAGE_SCALE<SCHEME> * (F - aq);
   }
 }
 
@@ -711,7 +719,7 @@ __global__ void __launch_bounds__(THREADS, SCHEME == IBFSA_MLP_TENO5 ? 4 : (CHAR
     float q[NV], fpv[NV], fmv[NV];
 #pragma unroll
     for (int c = 0; c < NV; c++) q[c] = p.Qp32[(size_t)c * p.NP + s];
-    split_cell<DIM, A>(fs, alpha, q, Wa[s], Wpr[s], fpv, fmv);
+    split_cell<DIM, A, PAIR ? SCHEME : -1>(fs, alpha, q, Wa[s], Wpr[s], fpv, fmv);
     if constexpr (ZL) {
 #pragma unroll
       for (int c = 0; c < NV; c++) {
@@ -807,7 +815,8 @@ __global__ void __launch_bounds__(THREADS, SCHEME == IBFSA_MLP_TENO5 ? 4 : (CHAR
     // and fi + 3: z_fi .. z_fi+4).  Every lane of the warp takes part (the slow path is warp-
     // uniform): lanes without a face evaluate a valid one and store nothing.
     static_assert(MAXP == 2, "two faces per thread");
-    int row = A == 0 ? warp : lane, fi = 2 * (A == 0 ? lane : warp);
+    static_assert(!PAIR || A != 0, "the x pass is k_conv32_x");
+    int row = lane, fi = 2 * warp;
     const bool v0 = row < nrow && fi < nface, v1 = row < nrow && fi + 1 < nface;
     if (!v0) fi = 0;
     if (row >= nrow) row = 0;
@@ -815,20 +824,10 @@ __global__ void __launch_bounds__(THREADS, SCHEME == IBFSA_MLP_TENO5 ? 4 : (CHAR
 #pragma unroll
     for (int c = 0; c < NV; c++) {
       float2 z[6];
-      if constexpr (A == 0) {  // 16-byte loads: fi and the row pitch are even
-        const float4 *z4 = reinterpret_cast<const float4 *>(zr + c * T::ROWS * T::LEN);
 #pragma unroll
-        for (int j = 0; j < 3; j++) {
-          const float4 v = z4[j];
-          z[2 * j] = make_float2(v.x, v.y);
-          z[2 * j + 1] = make_float2(v.z, v.w);
-        }
-      } else {
-#pragma unroll
-        for (int j = 0; j < 6; j++) z[j] = zr[c * T::ROWS * T::LEN + j];
-      }
+      for (int j = 0; j < 6; j++) z[j] = zr[c * T::ROWS * T::LEN + j];
       float h[2];
-      faces_pz2<SCHEME>(p, z, v0, v1, h);
+      faces_pz<SCHEME, 2>(p, z, v0, v1, h);
       Fh[0][c] = h[0];
       Fh[1][c] = h[1];
     }
@@ -839,7 +838,7 @@ __global__ void __launch_bounds__(THREADS, SCHEME == IBFSA_MLP_TENO5 ? 4 : (CHAR
   for (int ps = 0; ps < MAXP; ps++) {
     int e = threadIdx.x + ps * THREADS;
     int row, fi;
-    if constexpr (PAIR) { row = A == 0 ? warp : lane; fi = 2 * (A == 0 ? lane : warp) + ps; }
+    if constexpr (PAIR) { row = lane; fi = 2 * warp + ps; }
     else if constexpr (A == 0) { row = e / T::FACES; fi = e % T::FACES; }
     else { row = e % T::ROWS; fi = e / T::ROWS; }
     if (e < T::ROWS * T::FACES && row < nrow && fi < nface) {
@@ -867,13 +866,129 @@ __global__ void __launch_bounds__(THREADS, SCHEME == IBFSA_MLP_TENO5 ? 4 : (CHAR
     if (row >= nrow || l >= ncell) continue;
     int o = ibase + row * irs + l * ias;
     // the boundary cell of a characteristic face takes its normal term from k_char_face32
-    const float inv_h = char_cell(p, A, seg0 + l) ? 0.f : mesh::inv32(p, A, seg0 + l);
+    const float inv_h = char_cell(p, A, seg0 + l)
+                            ? 0.f : FLUX_SCALE<PAIR ? SCHEME : -1> * mesh::inv32(p, A, seg0 + l);
 #pragma unroll
     for (int c = 0; c < NV; c++) {
       const float *hh = sh + (c * T::ROWS + row) * FST;
       float d = (hh[l + 1] - hh[l]) * inv_h;
       float *Lc = p.L32 + (size_t)c * p.N;
       Lc[o] = (first ? 0.f : Lc[o]) - d;
+    }
+  }
+}
+
+// ------------------------------------------------------------------------------------------
+// x pass of the fixed component-wise schemes (the first pass: L' is written)
+// ------------------------------------------------------------------------------------------
+// LPR lanes per row of up to 2 LPR cells, two adjacent faces per lane; the rows of a block are
+// numbered through y and z.  After the staged split fluxes everything stays in the row's lanes:
+// the right face of a lane's second cell is its neighbour's first face (a shuffle), and that of a
+// full row's last cell is taken by the row's first NV lanes, one component each.  The last six
+// staged cells of all rows are staged together by a few warps.  One barrier, no face fluxes in
+// shared memory.
+// Against tiles of 63 cells whose face fluxes went through shared memory: TENO5 at 512^3 1.97 ->
+// 1.78 ms (eight rows of 64 instead of nine of 63, two barriers and 30 shared-memory accesses per
+// lane fewer); WENO5-JS at 2048^2 66.5 -> 64.8 us.  Five blocks per SM for TENO5 (1.81 ms with six,
+// which spill), six for WENO5-JS (69 us with five).
+template <int DIM, int LPR>
+struct RowTile {
+  static constexpr int NV = DIM + 2, CELLS = 2 * LPR, PITCH = CELLS + 6, RW = 32 / LPR;
+  static constexpr int ROWS = RW * THREADS / 32;
+  static constexpr size_t BYTES = sizeof(float2) * NV * ROWS * PITCH;
+};
+
+template <int DIM, int SCHEME, int LPR>
+__global__ void __launch_bounds__(THREADS, SCHEME == IBFSA_TENO5 ? 5 : 6) k_conv32_x(Plan p, int seg, int nseg) {
+  constexpr int NV = DIM + 2;
+  using T = RowTile<DIM, LPR>;
+  extern __shared__ __align__(16) float2 sz[];   // [NV][ROWS][PITCH]: z_l = (f+ at l, f- at l+1)
+  constexpr int SC = T::ROWS * T::PITCH;
+  const float alpha = (float)__longlong_as_double((long long)p.alpha_bits[0]);
+  const int lane = threadIdx.x & 31, sl = lane % LPR, row = (threadIdx.x >> 5) * T::RW + lane / LPR;
+  const int seg0 = (int)(blockIdx.x % nseg) * seg, row0 = (int)(blockIdx.x / nseg) * T::ROWS;
+  const int ncell = min(seg, p.n[0] - seg0), nface = ncell + 1, nrows = p.n[1] * p.n[2];
+  if (ncell <= 0) return;
+  const bool own = row0 + row < nrows;
+  // padded offset of staged cell 0 (cell seg0 - 3) of row r of the tile (rows past the end: the last)
+  auto padded = [&](int r) {
+    const int R = min(row0 + r, nrows - 1), z = R / p.n[1], y = R - z * p.n[1];
+    return ((z + p.g[2]) * p.P[1] + y + p.g[1]) * p.P[0] + seg0 + p.g[0] - 3;
+  };
+  const Free fs = free_stream(p);
+  const float *Wa = p.Wp32, *Wpr = p.Wp32 + (size_t)DIM * p.NP;
+  auto stage = [&](int r, int l, int s) {
+    float q[NV], fp[NV], fm[NV];
+#pragma unroll
+    for (int c = 0; c < NV; c++) q[c] = p.Qp32[(size_t)c * p.NP + s];
+    split_cell<DIM, 0, SCHEME>(fs, alpha, q, Wa[s], Wpr[s], fp, fm);
+    float2 *z = sz + r * T::PITCH + l;
+#pragma unroll
+    for (int c = 0; c < NV; c++) {
+      z[c * SC].x = fp[c];
+      if (l > 0) z[c * SC - 1].y = fm[c];
+    }
+  };
+  const int pb = padded(row);
+#pragma unroll
+  for (int k = 0; k < 2; k++) {
+    const int l = sl + k * LPR;
+    if (l < ncell + 6) stage(row, l, pb + l);
+  }
+  if (ncell + 6 > T::CELLS && threadIdx.x < 6 * T::ROWS) {
+    const int r = threadIdx.x / 6, l = T::CELLS + threadIdx.x % 6;
+    if (l < ncell + 6) stage(r, l, padded(r) + l);
+  }
+  __syncthreads();
+  const int fi = min(2 * sl, (nface - 1) & ~1);  // lanes past the last face repeat its pair
+  const bool v0 = own && 2 * sl < nface, v1 = own && 2 * sl + 1 < nface;
+  const float4 *z4 = reinterpret_cast<const float4 *>(sz + row * T::PITCH + fi);
+  float h0[NV], h1[NV], hn[NV];
+#pragma unroll
+  for (int c = 0; c < NV; c++) {
+    float2 z[6];
+#pragma unroll
+    for (int j = 0; j < 3; j++) {
+      const float4 v = z4[c * (SC / 2) + j];
+      z[2 * j] = make_float2(v.x, v.y);
+      z[2 * j + 1] = make_float2(v.z, v.w);
+    }
+    float h[2];
+    faces_pz<SCHEME, 2>(p, z, v0, v1, h);
+    h0[c] = h[0];
+    h1[c] = h[1];
+    hn[c] = __shfl_down_sync(0xffffffffu, h[0], 1, LPR);
+  }
+  if (ncell == T::CELLS) {  // the last face of a full row
+    float2 z[5];
+    const float2 *zl = sz + min(sl, NV - 1) * SC + row * T::PITCH + T::CELLS;
+#pragma unroll
+    for (int j = 0; j < 5; j++) z[j] = zl[j];
+    float h[1];
+    faces_pz<SCHEME, 1>(p, z, own && sl < NV, false, h);
+#pragma unroll
+    for (int c = 0; c < NV; c++) {
+      const float v = __shfl_sync(0xffffffffu, h[0], c, LPR);
+      if (sl == LPR - 1) hn[c] = v;
+    }
+  }
+  // L' = 0 - (Fhat_{m+1/2} - Fhat_{m-1/2}) / (dx/dxi) of cells 2 sl, 2 sl + 1; the boundary cell of
+  // a characteristic face takes its normal term from k_char_face32
+  const int l = 2 * sl, i = seg0 + l;
+  if (!own || l >= ncell) return;
+  const bool two = l + 1 < ncell;
+  const float inv0 = char_cell(p, 0, i) ? 0.f : FLUX_SCALE<SCHEME> * mesh::inv32(p, 0, i);
+  const float inv1 = !two || char_cell(p, 0, i + 1) ? 0.f : FLUX_SCALE<SCHEME> * mesh::inv32(p, 0, i + 1);
+  float *L = p.L32 + (size_t)(row0 + row) * p.n[0] + i;
+  const bool pair = two && !(p.n[0] & 1);  // 8-byte stores: rows and segments start at even cells
+#pragma unroll
+  for (int c = 0; c < NV; c++) {
+    const float d0 = 0.f - (h1[c] - h0[c]) * inv0, d1 = 0.f - (hn[c] - h1[c]) * inv1;
+    float *Lc = L + (size_t)c * p.N;
+    if (pair) *reinterpret_cast<float2 *>(Lc) = make_float2(d0, d1);
+    else {
+      Lc[0] = d0;
+      if (two) Lc[1] = d1;
     }
   }
 }
@@ -966,12 +1081,15 @@ __global__ void __launch_bounds__(THREADS, SCHEME == IBFSA_MLP_TENO5 ? 4 : 5)
   const float alpha = (float)__longlong_as_double((long long)p.alpha_bits[A]);
   {
     Free fs = free_stream(p);
-    for (int l = warp; l < ncell + 6; l += NW) {
+#pragma unroll
+    for (int k = 0; k < (LEN + NW - 1) / NW; k++) {
+      const int l = warp + k * NW;
+      if (l >= ncell + 6) break;
       float q[NV], fpv[NV], fmv[NV];
 #pragma unroll
       for (int c = 0; c < NV; c++) q[c] = in[(c * LEN + l) * R + lane];
-      split_cell<DIM, A>(fs, alpha, q, in[(NV * LEN + l) * R + lane],
-                         in[((NV + 1) * LEN + l) * R + lane], fpv, fmv);
+      split_cell<DIM, A, PAIR ? SCHEME : -1>(fs, alpha, q, in[(NV * LEN + l) * R + lane],
+                                             in[((NV + 1) * LEN + l) * R + lane], fpv, fmv);
       // interleaved face stencils z_l = (f+ at l, f- at l+1), [NV][LEN-1][R] float2
       float2 *Z = reinterpret_cast<float2 *>(sfp);
 #pragma unroll
@@ -1018,33 +1136,61 @@ __global__ void __launch_bounds__(THREADS, SCHEME == IBFSA_MLP_TENO5 ? 4 : 5)
 #pragma unroll
         for (int j = 0; j < 6; j++) z[j] = zc[j * R];
         float h[2];
-        faces_pz2<SCHEME>(p, z, row_ok, row_ok && fi + 1 < nface, h);
+        faces_pz<SCHEME, 2>(p, z, row_ok, row_ok && fi + 1 < nface, h);
         Fh[0][c] = h[0];
         Fh[1][c] = h[1];
       }
     }
   }
   __syncthreads();
-  float *sh = sfp;  // face fluxes [NV][R][FST]
-#pragma unroll
-  for (int ps = 0; ps < MAXP; ps++) {
-    const int fi = PAIR ? 2 * warp + ps : warp + ps * NW;
-    if (fi < nface) {
-#pragma unroll
-      for (int c = 0; c < NV; c++) sh[(c * R + lane) * FST + fi] = Fh[ps][c];
-    }
-  }
-  __syncthreads();
-  if (!block_wait_or_report(p, bar, 1)) return;
-
   // 3. L' = L' - (Fhat_{m+1/2} - Fhat_{m-1/2}) / (dx/dxi) on the copied tile, then stored back
-  if (row_ok) {
-    for (int l = warp; l < ncell; l += NW) {
-      const float inv_h = char_cell(p, A, seg0 + l) ? 0.f : mesh::inv32(p, A, seg0 + l);
+  auto inverse = [&](int l) {
+    return char_cell(p, A, seg0 + l) ? 0.f
+                                     : FLUX_SCALE<PAIR ? SCHEME : -1> * mesh::inv32(p, A, seg0 + l);
+  };
+  if constexpr (PAIR) {
+    // a warp owns faces 2 warp, 2 warp + 1 and the cells right of them; only the second cell's
+    // right face, the next warp's first, goes through shared memory (all of them before: with the
+    // staged fluxes' factor of a half left out, 2.22 -> 2.00 ms at 512^3)
+    float *sx = sfp;  // [NW][NV][R]
+    if (2 * warp < nface) {
 #pragma unroll
-      for (int c = 0; c < NV; c++) {
-        const float *hh = sh + (c * R + lane) * FST;
-        in[(c * SEG + l) * R + lane] -= (hh[l + 1] - hh[l]) * inv_h;
+      for (int c = 0; c < NV; c++) sx[(warp * NV + c) * R + lane] = Fh[0][c];
+    }
+    __syncthreads();
+    if (!block_wait_or_report(p, bar, 1)) return;
+    const int l = 2 * warp;
+    if (row_ok && l < ncell) {
+      const float i0 = inverse(l);
+#pragma unroll
+      for (int c = 0; c < NV; c++) in[(c * SEG + l) * R + lane] -= (Fh[1][c] - Fh[0][c]) * i0;
+      if (l + 1 < ncell) {
+        const float i1 = inverse(l + 1);
+#pragma unroll
+        for (int c = 0; c < NV; c++)
+          in[(c * SEG + l + 1) * R + lane] -= (sx[((warp + 1) * NV + c) * R + lane] - Fh[1][c]) * i1;
+      }
+    }
+  } else {
+    float *sh = sfp;  // face fluxes [NV][R][FST]
+#pragma unroll
+    for (int ps = 0; ps < MAXP; ps++) {
+      const int fi = warp + ps * NW;
+      if (fi < nface) {
+#pragma unroll
+        for (int c = 0; c < NV; c++) sh[(c * R + lane) * FST + fi] = Fh[ps][c];
+      }
+    }
+    __syncthreads();
+    if (!block_wait_or_report(p, bar, 1)) return;
+    if (row_ok) {
+      for (int l = warp; l < ncell; l += NW) {
+        const float inv_h = inverse(l);
+#pragma unroll
+        for (int c = 0; c < NV; c++) {
+          const float *hh = sh + (c * R + lane) * FST;
+          in[(c * SEG + l) * R + lane] -= (hh[l + 1] - hh[l]) * inv_h;
+        }
       }
     }
   }
@@ -1692,6 +1838,18 @@ cudaError_t conv_tensor_maps(const Plan &p, CUtensorMap *tq, CUtensorMap *tw, CU
   return tma::encode_f32_4d(tl, p.L32, dl, is, bl);
 }
 
+template <int DIM, int SCHEME, int LPR>
+cudaError_t launch_conv_x(const Plan &p, int nseg, cudaStream_t st) {
+  using T = RowTile<DIM, LPR>;
+  int seg = (p.n[0] + nseg - 1) / nseg;  // equal segments, starting at even cells
+  seg += seg & 1;
+  const long long rows = (long long)p.n[1] * p.n[2];
+  const long long blocks = (rows + T::ROWS - 1) / T::ROWS * nseg;
+  static_assert(T::BYTES <= 48 * 1024, "within the default dynamic shared memory");
+  k_conv32_x<DIM, SCHEME, LPR><<<(unsigned)blocks, THREADS, T::BYTES, st>>>(p, seg, nseg);
+  return cudaGetLastError();
+}
+
 template <int DIM, int A, int SCHEME>
 cudaError_t launch_conv(const Plan &p, int first, cudaStream_t st) {
   using T = Tile<A>;
@@ -1713,6 +1871,13 @@ cudaError_t launch_conv(const Plan &p, int first, cudaStream_t st) {
       return cudaGetLastError();
     }
   }
+  if constexpr (A == 0 && SCHEME != IBFSA_MLP_TENO5) {
+    // rows of 64 cells per warp, or of 32 (two rows per warp) where that leaves fewer empty slots
+    // (their halo of six cells costs ~5 % more)
+    const int n = p.n[0], wide = (n + 63) / 64, narrow = (n + 31) / 32;
+    return 64 * wide > 34 * narrow ? launch_conv_x<DIM, SCHEME, 16>(p, narrow, st)
+                                   : launch_conv_x<DIM, SCHEME, 32>(p, wide, st);
+  }
   if constexpr (A != 0) {
     if (p.n[0] % 4 == 0 && !first) {
       using TT = TmaTile<DIM, A>;
@@ -1730,6 +1895,7 @@ cudaError_t launch_conv(const Plan &p, int first, cudaStream_t st) {
       return cudaGetLastError();
     }
   }
+  if constexpr (A != 0 || SCHEME == IBFSA_MLP_TENO5) {
   constexpr size_t smem =
       conv_smem<DIM, A>() + (SCHEME == IBFSA_MLP_TENO5 ? (size_t)mlp::PACKED_BYTES : 0);
   e = cudaFuncSetAttribute(k_conv32<DIM, A, SCHEME>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1745,6 +1911,7 @@ cudaError_t launch_conv(const Plan &p, int first, cudaStream_t st) {
   }
   k_conv32<DIM, A, SCHEME><<<grid, THREADS, smem, st>>>(p, first);
   return cudaGetLastError();
+  }
 }
 
 // z-chunk of k_visc_march32.  A block's time is its planes (zc plus ~7 of start-up: the ring's
