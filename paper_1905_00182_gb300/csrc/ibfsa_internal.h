@@ -78,6 +78,16 @@ struct Plan {
   double *F;                  // marker force of Eq. 7 [dim][max_markers]
 };
 
+// cells of all characteristic faces (those of corners and edges once per face)
+inline long long char_cells(const Plan &p) {
+  long long cells = 0;
+  for (int a = 0; a < p.dim; a++)
+    for (int side = 0; side < 2; side++)
+      if (p.bc[a][side] == IBFSA_BC_CHARACTERISTIC)
+        cells += (long long)p.n[(a + 1) % 3] * p.n[(a + 2) % 3];
+  return cells;
+}
+
 // Kernel classes for launch counting and CUDA-event timing (instrumentation only).
 enum KClass {
   K_PAD = 0, K_INTERP, K_CONV_X, K_CONV_Y, K_CONV_Z, K_VISC_FLUX, K_VISC_DIV, K_SPREAD, K_FINISH,

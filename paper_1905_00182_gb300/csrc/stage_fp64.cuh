@@ -77,7 +77,7 @@ __device__ __forceinline__ int map_index(int i, int n, int rlo, int rhi) {
   return i;
 }
 
-// the boundary cell of a characteristic face along a (its normal term comes from k_char_face)
+// the boundary cell of a characteristic face along a (its normal term comes from k_char_faces)
 __device__ __forceinline__ bool char_cell(const Plan &p, int a, int i) {
   return (i == 0 && p.bc[a][0] == IBFSA_BC_CHARACTERISTIC) ||
          (i == p.n[a] - 1 && p.bc[a][1] == IBFSA_BC_CHARACTERISTIC);
@@ -753,7 +753,7 @@ __global__ void __launch_bounds__(THREADS) k_conv_char(Plan p, int first) {
     for (int c = 0; c < NV; c++) {
       const double *hh = sh + (c * T::ROWS + row) * FST;
       // dx/dxi at the cell (the spacing h on a uniform direction); the boundary cell of a
-      // characteristic face takes its normal term from k_char_face instead
+      // characteristic face takes its normal term from k_char_faces instead
       double d = char_cell(p, A, I[A]) ? 0.0
                  : p.mm[A] ? divide(hh[l + 1] - hh[l], p.mm[A][I[A] + NG], p.minv[A][I[A] + NG])
                            : divide(hh[l + 1] - hh[l], p.h[A], p.inv_h[A]);
@@ -888,7 +888,7 @@ __global__ void __launch_bounds__(THREADS, 3) k_conv(Plan p, int first, int nseg
   }
   __syncthreads();
   // 3. L = L - (Fhat_{m+1/2} - Fhat_{m-1/2}) / (dx/dxi); the boundary cell of a characteristic
-  // face takes its normal term from k_char_face instead.  A = 0: a warp walks the rows.
+  // face takes its normal term from k_char_faces instead.  A = 0: a warp walks the rows.
   constexpr int NW = THREADS / 32;
 #pragma unroll
   for (int i = 0; i < (A == 0 ? T::R / NW : (T::FACES + NW - 1) / NW); i++) {
@@ -927,18 +927,12 @@ __device__ __forceinline__ double one_sided(const double *phi, long long o, long
   return divide((double)s * acc, h12, inv_h12);
 }
 
-// one thread per cell of the face (a, side): L -= (dF_a/dx_a)_char, in the order the formulas
-// are written (the strict form reproduces a sequential evaluation)
+// the normal convective term (dF_a/dx_a)_char of the cell I on the face (a, side), in the order the
+// formulas are written (the strict form reproduces a sequential evaluation)
 template <int DIM>
-__global__ void k_char_face(Plan p, int a, int side) {
+__device__ __forceinline__ void char_term(const Plan &p, int a, int side, const int I[3],
+                                          double D[DIM + 2]) {
   constexpr int NV = DIM + 2;
-  const int b1 = (a + 1) % 3, b2 = (a + 2) % 3;
-  long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (long long)p.n[b1] * p.n[b2]) return;
-  int I[3];
-  I[a] = side == 0 ? 0 : p.n[a] - 1;
-  I[b1] = (int)(t % p.n[b1]);
-  I[b2] = (int)(t / p.n[b1]);
   const int s = side == 0 ? 1 : -1;
   const long long o = pad_index(p, I[0], I[1], I[2]);
   const long long st = a == 0 ? 1 : a == 1 ? (long long)p.P[0] : (long long)p.P[0] * p.P[1];
@@ -965,7 +959,6 @@ __global__ void k_char_face(Plan p, int a, int side) {
   const double d1 = (L2 + 0.5 * (L5 + L1)) / (c * c);
   const double d2 = 0.5 * (L5 + L1);
   dv[a] = (L5 - L1) / (2.0 * r * c);
-  double D[NV];
   double ke = 0.0, work = 0.0;
   D[0] = d1;
 #pragma unroll
@@ -976,9 +969,48 @@ __global__ void k_char_face(Plan p, int a, int side) {
     work = work + ub * dv[b];
   }
   D[NV - 1] = 0.5 * ke * d1 + d2 / p.gm1 + r * work;
-  const long long oi = int_index(p, I[0], I[1], I[2]);
+}
+
+// All characteristic faces in one launch, one thread per cell: the cell of a corner or an edge
+// belongs to the thread of its first face, which takes its faces' terms in order (direction by
+// direction, low face first).
+template <int DIM>
+__global__ void __launch_bounds__(128) k_char_faces(Plan p) {
+  constexpr int NV = DIM + 2;
+  long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  int I[3], face = -1;
 #pragma unroll
-  for (int c2 = 0; c2 < NV; c2++) p.L[c2 * p.N + oi] = p.L[c2 * p.N + oi] - D[c2];
+  for (int a = 0; a < DIM; a++)
+#pragma unroll
+    for (int side = 0; side < 2; side++) {
+      if (face >= 0 || p.bc[a][side] != IBFSA_BC_CHARACTERISTIC) continue;
+      const int b1 = (a + 1) % 3, b2 = (a + 2) % 3;
+      const long long cells = (long long)p.n[b1] * p.n[b2];
+      if (t < cells) {
+        face = 2 * a + side;
+        I[a] = side == 0 ? 0 : p.n[a] - 1;
+        I[b1] = (int)(t % p.n[b1]);
+        I[b2] = (int)(t / p.n[b1]);
+      }
+      t -= cells;
+    }
+  if (face < 0) return;
+  for (int a = 0; a < face / 2; a++)
+    if (char_cell(p, a, I[a])) return;  // another thread's cell
+  const long long oi = int_index(p, I[0], I[1], I[2]);
+  double L[NV];
+#pragma unroll
+  for (int c = 0; c < NV; c++) L[c] = p.L[c * p.N + oi];
+  for (int f = face; f < 2 * DIM; f++) {
+    const int a = f / 2, side = f % 2;
+    if (p.bc[a][side] != IBFSA_BC_CHARACTERISTIC || I[a] != (side == 0 ? 0 : p.n[a] - 1)) continue;
+    double D[NV];
+    char_term<DIM>(p, a, side, I, D);
+#pragma unroll
+    for (int c = 0; c < NV; c++) L[c] = L[c] - D[c];
+  }
+#pragma unroll
+  for (int c = 0; c < NV; c++) p.L[c * p.N + oi] = L[c];
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1570,16 +1602,12 @@ cudaError_t run_stage(const Plan &p, const StageArgs &s, cudaStream_t st) {
     prof_end(pr, K_CONV_Z, st);
     if (e != cudaSuccess) return e;
   }
-  // characteristic faces, direction by direction, low face first
-  for (int a = 0; a < DIM; a++)
-    for (int side = 0; side < 2; side++) {
-      if (p.bc[a][side] != IBFSA_BC_CHARACTERISTIC) continue;
-      long long cells = (long long)p.n[(a + 1) % 3] * p.n[(a + 2) % 3];
-      prof_begin(pr, st);
-      k_char_face<DIM><<<blocks_for(cells, THREADS), THREADS, 0, st>>>(p, a, side);
-      prof_end(pr, K_CONV_X + a, st);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
+  if (const long long cells = char_cells(p)) {
+    prof_begin(pr, st);
+    k_char_faces<DIM><<<blocks_for(cells, 128), 128, 0, st>>>(p);
+    prof_end(pr, K_CONV_X, st);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
   if (p.Re > 0.0) {
     prof_begin(pr, st);
     k_visc_flux<DIM><<<blocks_for(p.NB, THREADS), THREADS, 0, st>>>(p);
