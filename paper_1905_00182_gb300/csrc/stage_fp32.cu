@@ -566,6 +566,16 @@ __device__ __forceinline__ void split_cell(const Free &fs, float alpha, const fl
 // eigenvectors are the columns of R, left ones the rows of Lv, in the order u-c, entropy,
 // shears, u+c.  The split-flux perturbations are projected on them: their constant free-stream
 // part would pass through L and R unchanged and cancel in the face difference.
+// Whether entry c of left eigenvector k is zero whatever the state: the shears (k = 2 .. NV-2, one
+// per direction but A in increasing order) have entries for the density and their own momentum
+// only.  (Right eigenvectors: the momentum rows have the same zeros, the density row all shears'.)
+template <int DIM, int A>
+__host__ __device__ constexpr bool shear_zero(int k, int c) {
+  if (k < 2 || k > DIM || c == 0) return false;
+  const int t = k - 2, b = t < A ? t : t + 1;  // the shear's direction
+  return c != 1 + b;
+}
+
 template <int DIM, int A>
 __device__ __forceinline__ void roe_eigen32(const Free &fs, const float wl[DIM + 2],
                                             const float wr[DIM + 2], float R[DIM + 2][DIM + 2],
@@ -637,12 +647,15 @@ __device__ __forceinline__ void roe_eigen32(const Free &fs, const float wl[DIM +
   }
 }
 
-// Six blocks per SM (42 registers) for the fixed schemes' pairs of faces (x pass at 512^3 1.97 ms;
-// with 4 / 5 / 8 blocks 2.07 / 2.00 / 2.13), four (64 registers) for the learned form's warp-wide
-// network tiles, one for the characteristic-wise option (its two eigen-systems per face take
-// registers).  The x pass gives each warp one row of the tile.
+// Tiles by plain loads: the learned weights and the characteristic-wise option in every direction,
+// the fixed component-wise schemes along y and z where the x extent is not a multiple of 4.  Six
+// blocks per SM (42 registers) for the fixed schemes, four (64) for the learned form's warp-wide
+// network tiles.  The characteristic-wise option: four blocks for y and z, three for x (85
+// registers; four there spill and are 6 % slower); with one (138 registers, and each stencil
+// loaded and projected with the eigenvectors' zeros, field by field) a pass over 160 x 144 x 150
+// took 432 / 559 / 543 us, now 226 / 211 / 203 us.  The x pass gives each warp one row of the tile.
 template <int DIM, int A, int SCHEME, bool CHAR = false>
-__global__ void __launch_bounds__(THREADS, SCHEME == IBFSA_MLP_TENO5 ? 4 : (CHAR ? 1 : 6))
+__global__ void __launch_bounds__(THREADS, SCHEME == IBFSA_MLP_TENO5 ? 4 : (CHAR ? (A == 0 ? 3 : 4) : 6))
     k_conv32(Plan p, int first) {
   constexpr int NV = DIM + 2;
   using T = Tile<A>;
@@ -783,29 +796,42 @@ __global__ void __launch_bounds__(THREADS, SCHEME == IBFSA_MLP_TENO5 ? 4 : (CHAR
         }
         float Rm[NV][NV], Lv[NV][NV];
         roe_eigen32<DIM, A>(fs, wl, wr, Rm, Lv);
+        // one side after the other: its stencils of all components are loaded once (a load per
+        // field and component made 250 of them per face), and the eigenvectors' structural zeros
+        // (shear_zero) are skipped; each product sum in the order of the components
         float hk[NV];
 #pragma unroll
-        for (int k = 0; k < NV; k++) {
-          float vp[5], vm[5];
+        for (int k = 0; k < NV; k++) hk[k] = 0.f;
+#pragma unroll 1
+        for (int sd = 0; sd < 2; sd++) {
+          const float *f0 = (sd ? sfm + b + 3 : sfp + b - 2) + row * T::LEN;
+          const int st = sd ? -1 : 1;
+          float f[NV][5];
 #pragma unroll
-          for (int r = 0; r < 5; r++) {
-            float sp = 0.f, sn = 0.f;
+          for (int c = 0; c < NV; c++)
 #pragma unroll
-            for (int c = 0; c < NV; c++) {
-              sp = fmaf(Lv[k][c], sfp[(c * T::ROWS + row) * T::LEN + b - 2 + r], sp);
-              sn = fmaf(Lv[k][c], sfm[(c * T::ROWS + row) * T::LEN + b + 3 - r], sn);
+            for (int r = 0; r < 5; r++) f[c][r] = f0[c * T::ROWS * T::LEN + r * st];
+#pragma unroll
+          for (int k = 0; k < NV; k++) {
+            float v[5];
+#pragma unroll
+            for (int r = 0; r < 5; r++) {
+              float acc = 0.f;
+#pragma unroll
+              for (int c = 0; c < NV; c++)
+                if (!shear_zero<DIM, A>(k, c)) acc = fmaf(Lv[k][c], f[c][r], acc);
+              v[r] = acc;
             }
-            vp[r] = sp;
-            vm[r] = sn;
+            hk[k] += recon<SCHEME>(p, v[0], v[1], v[2], v[3], v[4]);
           }
-          hk[k] = recon<SCHEME>(p, vp[0], vp[1], vp[2], vp[3], vp[4]) +
-                  recon<SCHEME>(p, vm[0], vm[1], vm[2], vm[3], vm[4]);
         }
 #pragma unroll
         for (int c = 0; c < NV; c++) {
           float acc = 0.f;
 #pragma unroll
-          for (int k = 0; k < NV; k++) acc = fmaf(Rm[c][k], hk[k], acc);
+          for (int k = 0; k < NV; k++)
+            if (!(c == 0 ? k > 1 && k < NV - 1 : c < NV - 1 && shear_zero<DIM, A>(k, c)))
+              acc = fmaf(Rm[c][k], hk[k], acc);
           Fh[ps][c] = acc;
         }
       }
