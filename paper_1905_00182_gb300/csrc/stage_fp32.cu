@@ -753,16 +753,29 @@ __global__ void __launch_bounds__(THREADS, SCHEME == IBFSA_MLP_TENO5 ? 4 : (CHAR
   // 2. faces m+1/2, m = seg0-1 .. seg0+ncell-1 (tile face index fi = m - seg0 + 1)
   constexpr int MAXP = (T::ROWS * T::FACES + THREADS - 1) / THREADS;
   float Fh[MAXP][NV];
+  // the thread's face slot ps (row >= nrow or fi >= nface: none).  Learned weights along x: the
+  // tile's existing faces are numbered through its rows, so that a short last tile fills a few warps
+  // (the network costs a warp the same for one face as for 32): at 128^3, where the third tile of a
+  // row holds 2 of its 63 cells, the pass takes 868 us
+  // (1038 with the slots numbered through all 64 places of a row).
+  const unsigned face_magic = 65536u / nface + 1;  // e / nface for e < 512, nface <= 64
+  auto face_of = [&](int ps, int &row, int &fi) {
+    const int e = threadIdx.x + ps * THREADS;
+    if constexpr (PAIR) { row = lane; fi = 2 * warp + ps; }
+    else if constexpr (A == 0 && SCHEME == IBFSA_MLP_TENO5) {
+      row = (int)(e * face_magic >> 16);
+      fi = e - row * nface;
+    } else if constexpr (A == 0) { row = e / T::FACES; fi = e % T::FACES; }
+    else { row = e % T::ROWS; fi = e / T::ROWS; }
+  };
   if constexpr (SCHEME == IBFSA_MLP_TENO5) {
     unsigned char *img = reinterpret_cast<unsigned char *>(smf + 2 * NV * T::ROWS * T::LEN);
     unsigned used = 0, seen = 0;
     const float2 *Z = reinterpret_cast<const float2 *>(smf);
     learned_faces<MAXP, NV, 1>(p, img, Fh, used, seen, [&](int ps, int c, bool &valid) {
-      int e = threadIdx.x + ps * THREADS;
       int row, fi;
-      if constexpr (A == 0) { row = e / T::FACES; fi = e % T::FACES; }
-      else { row = e % T::ROWS; fi = e / T::ROWS; }
-      valid = e < T::ROWS * T::FACES && row < nrow && fi < nface;
+      face_of(ps, row, fi);
+      valid = row < nrow && fi < nface;
       if (!valid) { row = 0; fi = 0; }  // in-bounds reads; results discarded
       return Z + (c * T::ROWS + row) * T::LEN + fi;
     });
@@ -862,12 +875,9 @@ __global__ void __launch_bounds__(THREADS, SCHEME == IBFSA_MLP_TENO5 ? 4 : (CHAR
   float *sh = smf;
 #pragma unroll
   for (int ps = 0; ps < MAXP; ps++) {
-    int e = threadIdx.x + ps * THREADS;
     int row, fi;
-    if constexpr (PAIR) { row = lane; fi = 2 * warp + ps; }
-    else if constexpr (A == 0) { row = e / T::FACES; fi = e % T::FACES; }
-    else { row = e % T::ROWS; fi = e / T::ROWS; }
-    if (e < T::ROWS * T::FACES && row < nrow && fi < nface) {
+    face_of(ps, row, fi);
+    if (row < nrow && fi < nface) {
 #pragma unroll
       for (int c = 0; c < NV; c++) sh[(c * T::ROWS + row) * FST + fi] = Fh[ps][c];
     }
