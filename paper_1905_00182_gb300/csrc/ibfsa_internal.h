@@ -159,6 +159,7 @@ struct StageArgs {
   int stage;
   double src_scale;   // amp cos(omega t_stage) / (gamma - 1) of the pressure source (0: none)
   Prof *prof;
+  cudaEvent_t forces;  // recorded once the marker forces of the stage are known (NULL: not)
 };
 cudaError_t strict_stage(const Plan &p, const StageArgs &s, cudaStream_t st);
 cudaError_t fast_stage(const Plan &p, const StageArgs &s, cudaStream_t st);

@@ -1588,6 +1588,7 @@ cudaError_t run_stage(const Plan &p, const StageArgs &s, cudaStream_t st) {
     prof_end(pr, K_INTERP, st);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
+  if (s.forces && (e = cudaEventRecord(s.forces, st)) != cudaSuccess) return e;
   prof_begin(pr, st);
   e = launch_conv<DIM, 0, SCHEME>(p, 1, st);
   prof_end(pr, K_CONV_X, st);
