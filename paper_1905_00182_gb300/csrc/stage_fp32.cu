@@ -440,14 +440,12 @@ __device__ __forceinline__ float recon(const Plan &tw, float a, float b, float c
 template <int DIM>
 __global__ void __launch_bounds__(THREADS) k_pad32(Plan p, const float *__restrict__ din) {
   constexpr int NV = DIM + 2;
-  long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;  // padded cells fit in 31 bits
   float wmax[3] = {0.f, 0.f, 0.f};
-  if (t < p.NP) {
+  if (t < (unsigned)p.NP) {
     Free fs = free_stream(p);
-    int ix = (int)(t % p.P[0]);
-    long long r = t / p.P[0];
-    int iy = (int)(r % p.P[1]);
-    int iz = (int)(r / p.P[1]);
+    const unsigned r = t / (unsigned)p.P[0], rz = r / (unsigned)p.P[1];
+    const int ix = (int)(t - r * p.P[0]), iy = (int)(r - rz * p.P[1]), iz = (int)rz;
     int I[3] = {ix - p.g[0], iy - p.g[1], iz - p.g[2]};
     bool free_ghost = false, interior = true;
     int S[3];
@@ -1342,45 +1340,6 @@ __device__ __forceinline__ float d4f(float fm2, float fm1, float fp1, float fp2,
   return (8.f * (fp1 - fm1) - (fp2 - fm2)) * inv_h12;
 }
 
-template <int DIM>
-__global__ void __launch_bounds__(THREADS) k_visc_flux32(Plan p) {
-  long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= p.NB) return;
-  Free fs = free_stream(p);
-  int bx = (int)(t % p.B[0]);
-  long long r = t / p.B[0];
-  int by = (int)(r % p.B[1]);
-  int bz = (int)(r / p.B[1]);
-  int I[3] = {bx - 2, DIM > 1 ? by - 2 : by, DIM > 2 ? bz - 2 : bz};
-  long long s = pad_index(p, I[0], I[1], I[2]);
-  long long stride[3] = {1, p.P[0], (long long)p.P[0] * p.P[1]};
-  float g[DIM][DIM];
-#pragma unroll
-  for (int ci = 0; ci < DIM; ci++) {
-    const float *u = p.Wp32 + ci * p.NP + s;
-#pragma unroll
-    for (int dj = 0; dj < DIM; dj++) {
-      long long st = stride[dj];
-      g[ci][dj] = d4f(u[-2 * st], u[-st], u[st], u[2 * st], mesh::inv12_32(p, dj, I[dj]));
-    }
-  }
-  float div = 0.f;
-#pragma unroll
-  for (int a = 0; a < DIM; a++) div += g[a][a];
-#pragma unroll
-  for (int a = 0; a < DIM; a++) {
-    float b = 0.f;
-#pragma unroll
-    for (int ci = 0; ci < DIM; ci++) {
-      float tau = g[ci][a] + g[a][ci];
-      if (ci == a) tau -= (2.f / 3.f) * div;
-      p.V32[(long long)(a * (DIM + 1) + ci) * p.NB + t] = tau;
-      b += (fs.u[ci] + p.Wp32[ci * p.NP + s]) * tau;
-    }
-    p.V32[(long long)(a * (DIM + 1) + DIM) * p.NB + t] = b;
-  }
-}
-
 // ------------------------------------------------------------------------------------------
 // immersed boundary in FP64 from the FP64 stage state
 // ------------------------------------------------------------------------------------------
@@ -1475,44 +1434,17 @@ __device__ __forceinline__ float pressure_source32(const Plan &p, int dim, int i
   return expf(-(float)(p.src_b * 0.693147180559945309417) * r2) * (float)p.src_scale;
 }
 
-template <int DIM, bool VISC>
-__global__ void __launch_bounds__(THREADS) k_finish32(Plan p, const float *__restrict__ din,
-                                                      float *__restrict__ dout, double *Qn,
-                                                      double *__restrict__ Lout, float Bc,
-                                                      float dt, int mode) {
+// The end of a stage at one cell: sponge and pressure source on the right-hand side Lc of cell
+// (i, j, k), offset t, stage increment Dc, then the right-hand side out (mode 0) or the RK update
+template <int DIM, bool STRETCHED>
+__device__ __forceinline__ void finish_cell(const Plan &p, float (&Lc)[DIM + 2],
+                                            const float (&Dc)[DIM + 2], int i, int j, int k,
+                                            long long t, float *__restrict__ dout, double *Qn,
+                                            double *__restrict__ Lout, float Bc, float dt,
+                                            int mode) {
   constexpr int NV = DIM + 2;
-  long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= p.N) return;
-  float Lc[NV];
-#pragma unroll
-  for (int c = 0; c < NV; c++) Lc[c] = p.L32[c * p.N + t];
-  if constexpr (VISC) {
-    // viscous divergence (1/Re) sum_a D4_a [0, tau_{.a}, b_a], fused here to save a pass over L
-    int i = (int)(t % p.n[0]);
-    long long r = t / p.n[0];
-    int j = (int)(r % p.n[1]);
-    int k = (int)(r / p.n[1]);
-    long long bb = ((long long)(DIM > 2 ? k + 2 : k) * p.B[1] + (DIM > 1 ? j + 2 : j)) * p.B[0] + (i + 2);
-    long long stride[3] = {1, p.B[0], (long long)p.B[0] * p.B[1]};
-#pragma unroll
-    for (int fc = 0; fc <= DIM; fc++) {
-      float sum = 0.f;
-#pragma unroll
-      for (int a = 0; a < DIM; a++) {
-        const float *F = p.V32 + (long long)(a * (DIM + 1) + fc) * p.NB + bb;
-        long long st = stride[a];
-        sum += d4f(F[-2 * st], F[-st], F[st], F[2 * st],
-                   mesh::inv12_32(p, a, a == 0 ? i : a == 1 ? j : k));
-      }
-      Lc[fc + 1] += sum * p.inv_Re32;
-    }
-  }
   if (p.sponge_cells > 0) {
-    int I[3];
-    I[0] = (int)(t % p.n[0]);
-    long long r = t / p.n[0];
-    I[1] = (int)(r % p.n[1]);
-    I[2] = (int)(r / p.n[1]);
+    const int I[3] = {i, j, k};
     int S = p.sponge_cells, nmin = 1 << 30;
 #pragma unroll
     for (int a = 0; a < DIM; a++) nmin = min(nmin, min(I[a], p.n[a] - 1 - I[a]));
@@ -1520,17 +1452,10 @@ __global__ void __launch_bounds__(THREADS) k_finish32(Plan p, const float *__res
       float rr = (float)(S - nmin) / (float)S;
       float sig = (float)p.sponge_sigma * rr * rr * rr;
 #pragma unroll
-      for (int c = 0; c < NV; c++) {
-        float qp = p.qn32[c * p.N + t] + (din ? din[c * p.N + t] : 0.f);
-        Lc[c] -= sig * qp;
-      }
+      for (int c = 0; c < NV; c++) Lc[c] -= sig * (p.qn32[c * p.N + t] + Dc[c]);
     }
   }
-  if (p.src_on) {
-    int i = (int)(t % p.n[0]);
-    long long r = t / p.n[0];
-    Lc[NV - 1] += pressure_source32(p, DIM, i, (int)(r % p.n[1]), (int)(r / p.n[1]));
-  }
+  if (p.src_on) Lc[NV - 1] += pressure_source32<STRETCHED>(p, DIM, i, j, k);
   if (mode == 0) {
 #pragma unroll
     for (int c = 0; c < NV; c++) Lout[c * p.N + t] = (double)Lc[c];
@@ -1540,7 +1465,7 @@ __global__ void __launch_bounds__(THREADS) k_finish32(Plan p, const float *__res
   float inc[NV];
 #pragma unroll
   for (int c = 0; c < NV; c++) {
-    inc[c] = Bc * ((din ? din[c * p.N + t] : 0.f) + dt * Lc[c]);
+    inc[c] = Bc * (Dc[c] + dt * Lc[c]);
     bad |= !isfinite(inc[c]);
   }
   if (mode == 1) {
@@ -1555,6 +1480,147 @@ __global__ void __launch_bounds__(THREADS) k_finish32(Plan p, const float *__res
     }
   }
   if (bad) atomicOr(p.status, IBFSA_STATUS_NONFINITE);
+}
+
+// inviscid: one thread per cell
+template <int DIM>
+__global__ void __launch_bounds__(THREADS) k_finish32(Plan p, const float *__restrict__ din,
+                                                      float *__restrict__ dout, double *Qn,
+                                                      double *__restrict__ Lout, float Bc,
+                                                      float dt, int mode) {
+  constexpr int NV = DIM + 2;
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;  // cells fit in 31 bits
+  if (t >= (unsigned)p.N) return;
+  float Lc[NV], Dc[NV];
+#pragma unroll
+  for (int c = 0; c < NV; c++) {
+    Lc[c] = p.L32[c * p.N + t];
+    Dc[c] = din ? din[c * p.N + t] : 0.f;
+  }
+  const unsigned r = t / (unsigned)p.n[0], k = r / (unsigned)p.n[1];
+  finish_cell<DIM, true>(p, Lc, Dc, (int)(t - r * p.n[0]), (int)(r - k * p.n[1]), (int)k, t, dout,
+                         Qn, Lout, Bc, dt, mode);
+}
+
+// 2D viscous term + finish.  A block of 256 threads owns 64 x 16 cells: the velocity perturbations
+// with a halo of four in shared memory, from them the viscous fluxes at the block's cells and at the
+// two halo points per side that the divergence needs, in shared memory, then the divergence, sponge
+// and RK update.  The right-hand side and the stage increment are loaded while the fluxes are
+// evaluated.  Before, a kernel wrote the six flux arrays and the finish pass read them (48 B of
+// 136 per cell and stage) and both found their cell by 64-bit divisions:
+// together 132 -> 85 us per stage at 2048^2 and 244 -> 157 us at 4096 x 2048 (event times).
+namespace v2 {
+constexpr int TX = 64, TY = 16, PER = TX * TY / THREADS;  // cells of a block, per thread
+constexpr int SX = TX + 8, SY = TY + 8;                   // staged points
+constexpr int FX = TX + 4, FY = TY + 4;                   // points of F_v,x and F_v,y
+constexpr size_t SMEM = sizeof(float) * (2 * SX * SY + 3 * FX * TY + 3 * TX * FY);
+}  // namespace v2
+
+template <bool STRETCHED>
+__global__ void __launch_bounds__(THREADS, 4) k_visc_finish32(Plan p, const float *__restrict__ din,
+                                                           float *__restrict__ dout, double *Qn,
+                                                           double *__restrict__ Lout, float Bc,
+                                                           float dt, int mode) {
+  using namespace v2;
+  extern __shared__ float smm[];
+  float *su = smm, *sv = su + SX * SY;            // [SY][SX]
+  float *fx = sv + SX * SY, *fy = fx + 3 * FX * TY;  // [3][TY][FX], [3][FY][TX]
+  const int tx = threadIdx.x % TX, tq = threadIdx.x / TX;
+  constexpr int RS = THREADS / TX;                // rows tq, tq + RS, ...
+  const int tiles_x = (p.n[0] + TX - 1) / TX;
+  const int x0 = (int)(blockIdx.x % tiles_x) * TX, y0 = (int)(blockIdx.x / tiles_x) * TY;
+  const int X = x0 + tx;
+  const Free fs = free_stream(p);
+  const float *W0 = p.Wp32, *W1 = p.Wp32 + p.NP;
+#pragma unroll
+  for (int e = threadIdx.x; e < SX * SY; e += THREADS) {
+    const int sx = e % SX, sy = e / SX;
+    const int gx = min(x0 - 4 + sx, p.n[0] + 3), gy = min(y0 - 4 + sy, p.n[1] + 3);
+    const int o = (gy + p.g[1]) * p.P[0] + gx + p.g[0];
+    su[e] = W0[o];
+    sv[e] = W1[o];
+  }
+  float L[PER][4], D[PER][4];
+#pragma unroll
+  for (int k = 0; k < PER; k++) {
+    const int Y = y0 + tq + k * RS;
+    if (X < p.n[0] && Y < p.n[1]) {
+      const int t = Y * p.n[0] + X;
+#pragma unroll
+      for (int c = 0; c < 4; c++) {
+        L[k][c] = p.L32[c * p.N + t];
+        D[k][c] = din ? din[c * p.N + t] : 0.f;
+      }
+    }
+  }
+  __syncthreads();
+  // 1/(12 dx/dxi) of node i along a; indices of staged points beyond the box (their results are
+  // never used) are clamped into it
+  auto ihat = [&](int a, int i) -> float {
+    if constexpr (STRETCHED)
+      return p.minv12_32[a] ? p.minv12_32[a][mesh::clamp_node(p, a, i) + NG] : p.inv_h12_32[a];
+    else
+      return p.inv_h12_32[a];
+  };
+  // viscous fluxes at tile position (px, py), -2 .. TX+1 and -2 .. TY+1: [tau_0a, tau_1a, b_a]
+  auto flux = [&](int px, int py, bool wx, bool wy) {
+    const float ihx = ihat(0, x0 + px), ihy = ihat(1, y0 + py);
+    const int e = (py + 4) * SX + px + 4;
+    const float *m[2] = {su + e, sv + e};
+    float g[2][2];
+#pragma unroll
+    for (int i = 0; i < 2; i++) {
+      g[i][0] = d4f(m[i][-2], m[i][-1], m[i][1], m[i][2], ihx);
+      g[i][1] = d4f(m[i][-2 * SX], m[i][-SX], m[i][SX], m[i][2 * SX], ihy);
+    }
+    const float div = g[0][0] + g[1][1];
+#pragma unroll
+    for (int a = 0; a < 2; a++) {
+      if (a == 0 ? !wx : !wy) continue;
+      float *F = a == 0 ? fx + py * FX + px + 2 : fy + (py + 2) * TX + px;
+      const int st = a == 0 ? FX * TY : TX * FY;
+      float b = 0.f;
+#pragma unroll
+      for (int i = 0; i < 2; i++) {
+        float tau = g[i][a] + g[a][i];
+        if (i == a) tau -= (2.f / 3.f) * div;
+        F[i * st] = tau;
+        b += (fs.u[i] + m[i][0]) * tau;
+      }
+      F[2 * st] = b;
+    }
+  };
+#pragma unroll
+  for (int k = 0; k < PER; k++) flux(tx, tq + k * RS, true, true);
+  flux(tx, tq < 2 ? tq - 2 : TY + tq - 2, false, true);  // y halo: four rows of TX points
+  if (threadIdx.x < 4 * TY) {                               // x halo: four columns of TY points
+    const int h = threadIdx.x % 4;
+    flux(h < 2 ? h - 2 : TX + h - 2, threadIdx.x / 4, true, false);
+  }
+  __syncthreads();
+  const float ihx = ihat(0, X);
+#pragma unroll
+  for (int k = 0; k < PER; k++) {
+    const int py = tq + k * RS, Y = y0 + py;
+    if (X >= p.n[0] || Y >= p.n[1]) continue;
+    const float ihy = ihat(1, Y);
+    float Lc[4], Dc[4];
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+      Lc[c] = L[k][c];
+      Dc[c] = D[k][c];
+    }
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+      const float *Fx = fx + (c * TY + py) * FX + tx + 2, *Fy = fy + (c * FY + py + 2) * TX + tx;
+      float sum = 0.f;
+      sum += d4f(Fx[-2], Fx[-1], Fx[1], Fx[2], ihx);
+      sum += d4f(Fy[-2 * TX], Fy[-TX], Fy[TX], Fy[2 * TX], ihy);
+      Lc[c + 1] += sum * p.inv_Re32;
+    }
+    finish_cell<2, STRETCHED>(p, Lc, Dc, X, Y, 0, (long long)Y * p.n[0] + X, dout, Qn, Lout, Bc, dt,
+                              mode);
+  }
 }
 
 // 3D viscous term + finish, marching along z.  A 32 x 8 block of threads owns 32 x 8 columns
@@ -1789,43 +1855,7 @@ __global__ void __launch_bounds__(vm::VT, VM_MIN_BLOCKS) k_visc_march32(Plan p, 
       for (int cc = 0; cc < 5; cc++) Lc[cc] = Lnext[cc];
 #pragma unroll
       for (int k = 0; k < 4; k++) Lc[k + 1] += acc[0][k] * p.inv_Re32;
-      if (p.sponge_cells > 0) {
-        int I[3] = {X, Y, d};
-        int S = p.sponge_cells, nmin = 1 << 30;
-#pragma unroll
-        for (int a = 0; a < 3; a++) nmin = min(nmin, min(I[a], p.n[a] - 1 - I[a]));
-        if (nmin < S) {
-          float rr = (float)(S - nmin) / (float)S;
-          float sig = (float)p.sponge_sigma * rr * rr * rr;
-#pragma unroll
-          for (int cc = 0; cc < 5; cc++) Lc[cc] -= sig * (p.qn32[cc * p.N + t] + Dnext[cc]);
-        }
-      }
-      if (p.src_on) Lc[4] += pressure_source32<STRETCHED>(p, 3, X, Y, d);
-      if (mode == 0) {
-#pragma unroll
-        for (int cc = 0; cc < 5; cc++) Lout[cc * p.N + t] = (double)Lc[cc];
-      } else {
-        bool bad = false;
-        float inc[5];
-#pragma unroll
-        for (int cc = 0; cc < 5; cc++) {
-          inc[cc] = Bc * (Dnext[cc] + dt * Lc[cc]);
-          bad |= !isfinite(inc[cc]);
-        }
-        if (mode == 1) {
-#pragma unroll
-          for (int cc = 0; cc < 5; cc++) dout[cc * p.N + t] = inc[cc];
-        } else {
-#pragma unroll
-          for (int cc = 0; cc < 5; cc++) {
-            double qv = Qn[cc * p.N + t] + (double)inc[cc];
-            Qn[cc * p.N + t] = qv;
-            p.qn32[cc * p.N + t] = (float)(qv - p.qinf[cc]);
-          }
-        }
-        if (bad) atomicOr(p.status, IBFSA_STATUS_NONFINITE);
-      }
+      finish_cell<3, STRETCHED>(p, Lc, Dnext, X, Y, d, t, dout, Qn, Lout, Bc, dt, mode);
     }
     // plane c + 3 (needed from the next iteration on) replaces plane c - 2, whose gradients
     // were all taken before the barrier above; plane c + 4 starts loading
@@ -2050,12 +2080,6 @@ cudaError_t run_stage(const Plan &p, const StageArgs &s, cudaStream_t st) {
     prof_end(pr, K_CONV_X, st);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  if (p.Re > 0.0 && DIM == 2) {
-    prof_begin(pr, st);
-    k_visc_flux32<DIM><<<blocks_for(p.NB, THREADS), THREADS, 0, st>>>(p);
-    prof_end(pr, K_VISC_FLUX, st);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
   if (p.nm > 0) {
     prof_begin(pr, st);
     k_spread32<DIM><<<blocks_for((long long)p.nm * marker::Support<DIM>::G, 128), 128, 0, st>>>(
@@ -2077,12 +2101,18 @@ cudaError_t run_stage(const Plan &p, const StageArgs &s, cudaStream_t st) {
     dim3 grid((p.n[0] + TX - 1) / TX, (p.n[1] + TY - 1) / TY, (p.n[2] + zc - 1) / zc);
     kern<<<grid, VT, SMEM, st>>>(q, din, dout, const_cast<double *>(Qn), s.Lout, (float)s.b,
                                  (float)s.dt, mode, zc);
-  } else if (p.Re > 0.0)
-    k_finish32<DIM, true><<<blocks_for(p.N, THREADS), THREADS, 0, st>>>(
+  } else if (p.Re > 0.0) {
+    using namespace v2;
+    const bool stretched = p.minv12_32[0] || p.minv12_32[1];
+    auto kern = stretched ? k_visc_finish32<true> : k_visc_finish32<false>;
+    static_assert(SMEM <= 48 * 1024, "within the default dynamic shared memory");
+    const unsigned tiles = (unsigned)((p.n[0] + TX - 1) / TX) * ((p.n[1] + TY - 1) / TY);
+    kern<<<tiles, THREADS, SMEM, st>>>(q, din, dout, const_cast<double *>(Qn), s.Lout, (float)s.b,
+                                       (float)s.dt, mode);
+  } else {
+    k_finish32<DIM><<<blocks_for(p.N, THREADS), THREADS, 0, st>>>(
         q, din, dout, const_cast<double *>(Qn), s.Lout, (float)s.b, (float)s.dt, mode);
-  else
-    k_finish32<DIM, false><<<blocks_for(p.N, THREADS), THREADS, 0, st>>>(
-        q, din, dout, const_cast<double *>(Qn), s.Lout, (float)s.b, (float)s.dt, mode);
+  }
   prof_end(pr, K_FINISH, st);
   return cudaGetLastError();
 }
