@@ -31,6 +31,22 @@ constexpr int OFF_B2 = 10880;
 constexpr int OFF_B3 = 11008;
 constexpr int OFF_B4 = 11136;    // [8] f32
 constexpr int PACKED_BYTES = 11264;
+// The same image in a block's shared memory: the zero columns 8..15 of W1 and W4T left out (16-byte
+// rows), rows of 32 columns padded to 80 bytes.  A fragment load touches 8 rows x 4 words: at a
+// row stride of 64 bytes they met in 8 of 32 banks, at 16 and at 80 bytes in 32.
+constexpr int LD8 = 8, LD32 = 40;
+constexpr int S_W1 = 0;                  // [32][8]
+constexpr int S_W4T = 512;               // [32][8]
+constexpr int S_W2 = 1024;               // [32][40]
+constexpr int S_W3 = S_W2 + 2560;        // [32][40]
+constexpr int S_W2T = S_W3 + 2560;       // [32][40]
+constexpr int S_W3T = S_W2T + 2560;      // [32][40]
+constexpr int S_W4 = S_W3T + 2560;       // [8][40]
+constexpr int S_B1 = S_W4 + 640;         // [32] f32
+constexpr int S_B2 = S_B1 + 128;
+constexpr int S_B3 = S_B2 + 128;
+constexpr int S_B4 = S_B3 + 128;         // [8] f32
+constexpr int STAGED_BYTES = S_B4 + 32;
 // offsets of the flat parameter vector [W1 (32x5), b1, W2, b2, W3, b3, W4 (3x32), b4]
 constexpr int P_W1 = 0, P_B1 = 160, P_W2 = 192, P_B2 = 1216, P_W3 = 1248, P_B3 = 2272,
               P_W4 = 2304, P_B4 = 2400;
@@ -52,13 +68,22 @@ __device__ __forceinline__ void mma16816(float d[4], const uint32_t a[4], uint32
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-__device__ __forceinline__ float gelu(float z) {
-  return 0.5f * z * (1.f + tanhf(GELU_K * (z + GELU_C * z * z * z)));
+// the product over 8 inputs only
+__device__ __forceinline__ void mma1688(float d[4], uint32_t a0, uint32_t a1, uint32_t b0) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k8.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, "
+      "{%0,%1,%2,%3};\n"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a0), "r"(a1), "r"(b0));
 }
 
-__device__ __forceinline__ float gelu_grad(float z) {
-  float t = tanhf(GELU_K * (z + GELU_C * z * z * z));
-  return 0.5f * (1.f + t) + 0.5f * z * (1.f - t * t) * GELU_K * (1.f + 3.f * GELU_C * z * z);
+// gelu of z; with GRAD, z becomes the derivative there (the same tanh serves both)
+template <bool GRAD>
+__device__ __forceinline__ float gelu(float &z) {
+  const float t = tanhf(GELU_K * (z + GELU_C * z * z * z)), a = 0.5f * z * (1.f + t);
+  if (GRAD)
+    z = 0.5f * (1.f + t) + 0.5f * z * (1.f - t * t) * GELU_K * (1.f + 3.f * GELU_C * z * z);
+  return a;
 }
 
 // 32-bit load of two consecutive bf16 of a packed matrix with `ld` columns
@@ -71,79 +96,105 @@ __device__ __forceinline__ float ldb(const unsigned char *img, int off, int i) {
   return reinterpret_cast<const float *>(img + off)[i];
 }
 
+// the image's shared copy; a barrier has to follow
+__device__ __forceinline__ void stage_image(unsigned char *img,
+                                            const unsigned char *__restrict__ gimg) {
+  constexpr int CHUNKS = PACKED_BYTES / 16;
+  for (int i = threadIdx.x; i < CHUNKS; i += blockDim.x) {
+    const int b = 16 * i;
+    int to;
+    if (b < OFF_W2) {
+      if (i & 1) continue;
+      to = S_W1 + b / 2;
+    } else if (b < OFF_W2T) {  // W2, W3, W4: rows of 64 bytes
+      const int r = (b - OFF_W2) / 64;
+      to = (r < 32 ? S_W2 + 80 * r : r < 64 ? S_W3 + 80 * (r - 32) : S_W4 + 80 * (r - 64)) + b % 64;
+    } else if (b < OFF_W4T) {  // W2T, W3T
+      const int r = (b - OFF_W2T) / 64;
+      to = S_W2T + 80 * r + (b - OFF_W2T) % 64;
+    } else if (b < OFF_B1) {
+      if (i & 1) continue;
+      to = S_W4T + (b - OFF_W4T) / 2;
+    } else {
+      if (b >= OFF_B4 + 32) continue;
+      to = S_B1 + (b - OFF_B1);
+    }
+    *reinterpret_cast<uint4 *>(img + to) = reinterpret_cast<const uint4 *>(gimg)[i];
+  }
+}
+
 // 16x32 hidden layer: acc[j][.] (n-tile j = units 8j..8j+7) = bias + A(16 x K) W^T
-template <int KSTEPS>
-__device__ __forceinline__ void dense32(float acc[4][4], const uint32_t A[KSTEPS][4],
-                                        const unsigned char *img, int offW, int ldW, int offB,
-                                        int g, int t) {
+__device__ __forceinline__ void dense32(float acc[4][4], const uint32_t A[2][4],
+                                        const unsigned char *img, int offW, int offB, int g,
+                                        int t) {
 #pragma unroll
   for (int j = 0; j < 4; j++) {
     float b0 = ldb(img, offB, 8 * j + 2 * t), b1 = ldb(img, offB, 8 * j + 2 * t + 1);
     acc[j][0] = b0; acc[j][1] = b1; acc[j][2] = b0; acc[j][3] = b1;
 #pragma unroll
-    for (int s = 0; s < KSTEPS; s++) {
-      uint32_t w0 = ldw(img, offW, ldW, 8 * j + g, 16 * s + 2 * t);
-      uint32_t w1 = ldw(img, offW, ldW, 8 * j + g, 16 * s + 2 * t + 8);
+    for (int s = 0; s < 2; s++) {
+      uint32_t w0 = ldw(img, offW, LD32, 8 * j + g, 16 * s + 2 * t);
+      uint32_t w1 = ldw(img, offW, LD32, 8 * j + g, 16 * s + 2 * t + 8);
       mma16816(acc[j], A[s], w0, w1);
     }
   }
 }
 
-// gelu of a 16x32 accumulator, packed as the next layer's two BF16 k-step fragments
-__device__ __forceinline__ void gelu_pack(const float z[4][4], uint32_t A[2][4]) {
+// the first layer, inputs 0..7 of A0 (5 used)
+__device__ __forceinline__ void dense8(float acc[4][4], const uint32_t A0[2],
+                                       const unsigned char *img, int g, int t) {
 #pragma unroll
-  for (int s = 0; s < 2; s++) {
-    A[s][0] = pack2(gelu(z[2 * s][0]), gelu(z[2 * s][1]));
-    A[s][1] = pack2(gelu(z[2 * s][2]), gelu(z[2 * s][3]));
-    A[s][2] = pack2(gelu(z[2 * s + 1][0]), gelu(z[2 * s + 1][1]));
-    A[s][3] = pack2(gelu(z[2 * s + 1][2]), gelu(z[2 * s + 1][3]));
+  for (int j = 0; j < 4; j++) {
+    float b0 = ldb(img, S_B1, 8 * j + 2 * t), b1 = ldb(img, S_B1, 8 * j + 2 * t + 1);
+    acc[j][0] = b0; acc[j][1] = b1; acc[j][2] = b0; acc[j][3] = b1;
+    mma1688(acc[j], A0[0], A0[1], ldw(img, S_W1, LD8, 8 * j + g, 2 * t));
   }
+}
+
+// gelu of a 16x32 accumulator, packed as the next layer's two BF16 k-step fragments
+template <bool GRAD>
+__device__ __forceinline__ void gelu_pack(float z[4][4], uint32_t A[2][4]) {
+#pragma unroll
+  for (int s = 0; s < 2; s++)
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+      float *r = z[2 * s + h];
+      const float a0 = gelu<GRAD>(r[0]), a1 = gelu<GRAD>(r[1]);
+      const float a2 = gelu<GRAD>(r[2]), a3 = gelu<GRAD>(r[3]);
+      A[s][2 * h] = pack2(a0, a1);
+      A[s][2 * h + 1] = pack2(a2, a3);
+    }
 }
 
 // input fragment of layer 1 from the normalised stencils of rows g (xa) and g+8 (xb)
 __device__ __forceinline__ void input_fragment(const float xa[5], const float xb[5], int t,
-                                               uint32_t A[1][4]) {
+                                               uint32_t A[2]) {
   float a0 = 0.f, a1 = 0.f, b0 = 0.f, b1 = 0.f;
   if (t == 0) { a0 = xa[0]; a1 = xa[1]; b0 = xb[0]; b1 = xb[1]; }
   if (t == 1) { a0 = xa[2]; a1 = xa[3]; b0 = xb[2]; b1 = xb[3]; }
   if (t == 2) { a0 = xa[4]; b0 = xb[4]; }
-  A[0][0] = pack2(a0, a1);
-  A[0][1] = pack2(b0, b1);
-  A[0][2] = 0u;
-  A[0][3] = 0u;
+  A[0] = pack2(a0, a1);
+  A[1] = pack2(b0, b1);
 }
 
 // logits of layer 4 (16 x 8 accumulator, logits 0..2 used)
 __device__ __forceinline__ void logits(float z4[4], const uint32_t A3[2][4],
                                        const unsigned char *img, int g, int t) {
-  z4[0] = ldb(img, OFF_B4, 2 * t);
-  z4[1] = ldb(img, OFF_B4, 2 * t + 1);
+  z4[0] = ldb(img, S_B4, 2 * t);
+  z4[1] = ldb(img, S_B4, 2 * t + 1);
   z4[2] = z4[0];
   z4[3] = z4[1];
 #pragma unroll
   for (int s = 0; s < 2; s++) {
-    uint32_t w0 = ldw(img, OFF_W4, 32, g, 16 * s + 2 * t);
-    uint32_t w1 = ldw(img, OFF_W4, 32, g, 16 * s + 2 * t + 8);
+    uint32_t w0 = ldw(img, S_W4, LD32, g, 16 * s + 2 * t);
+    uint32_t w1 = ldw(img, S_W4, LD32, g, 16 * s + 2 * t + 8);
     mma16816(z4, A3[s], w0, w1);
   }
 }
 
-// Full forward of one 16-row tile.  On return, lanes with t == 0 hold the three softmax
-// weights of rows g (wa) and g+8 (wb).  z1..z3 keep the pre-activations for a backward pass.
-__device__ __forceinline__ void forward_tile(const unsigned char *img, const float xa[5],
-                                             const float xb[5], int g, int t, float z1[4][4],
-                                             float z2[4][4], float z3[4][4], uint32_t A1[2][4],
-                                             uint32_t A2[2][4], uint32_t A3[2][4], float wa[3],
-                                             float wb[3], float z4[4]) {
-  uint32_t A0[1][4];
-  input_fragment(xa, xb, t, A0);
-  dense32<1>(z1, A0, img, OFF_W1, 16, OFF_B1, g, t);
-  gelu_pack(z1, A1);
-  dense32<2>(z2, A1, img, OFF_W2, 32, OFF_B2, g, t);
-  gelu_pack(z2, A2);
-  dense32<2>(z3, A2, img, OFF_W3, 32, OFF_B3, g, t);
-  gelu_pack(z3, A3);
-  logits(z4, A3, img, g, t);
+// Softmax over the logits of a 16-row tile: lanes with t == 0 get the three weights of rows g (wa)
+// and g+8 (wb).
+__device__ __forceinline__ void softmax3(const float z4[4], float wa[3], float wb[3]) {
   // logits 0,1 live in lane t = 0, logit 2 in lane t = 1 (c0 / c2 for rows g / g+8)
   float l2a = __shfl_down_sync(0xffffffffu, z4[0], 1);
   float l2b = __shfl_down_sync(0xffffffffu, z4[2], 1);
