@@ -26,6 +26,7 @@
 #include <stdint.h>
 
 #include "ibfsa_internal.h"
+#include "launch.cuh"
 #include "marker.cuh"
 #include "mesh.cuh"
 #include "mlp_tile.cuh"
@@ -439,6 +440,7 @@ __device__ __forceinline__ float recon(const Plan &tw, float a, float b, float c
 // ------------------------------------------------------------------------------------------
 template <int DIM>
 __global__ void __launch_bounds__(THREADS) k_pad32(Plan p, const float *__restrict__ din) {
+  begin_kernel();
   constexpr int NV = DIM + 2;
   const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;  // padded cells fit in 31 bits
   float wmax[3] = {0.f, 0.f, 0.f};
@@ -655,6 +657,7 @@ __device__ __forceinline__ void roe_eigen32(const Free &fs, const float wl[DIM +
 template <int DIM, int A, int SCHEME, bool CHAR = false>
 __global__ void __launch_bounds__(THREADS, SCHEME == IBFSA_MLP_TENO5 ? 4 : (CHAR ? (A == 0 ? 3 : 4) : 6))
     k_conv32(Plan p, int first) {
+  begin_kernel();
   constexpr int NV = DIM + 2;
   using T = Tile<A>;
   static_assert(A != 0 || T::ROWS * 32 == THREADS, "x pass: one warp per row");
@@ -934,6 +937,7 @@ struct RowTile {
 
 template <int DIM, int SCHEME, int LPR>
 __global__ void __launch_bounds__(THREADS, SCHEME == IBFSA_TENO5 ? 5 : 6) k_conv32_x(Plan p, int seg, int nseg) {
+  begin_kernel();
   constexpr int NV = DIM + 2;
   using T = RowTile<DIM, LPR>;
   extern __shared__ __align__(16) float2 sz[];   // [NV][ROWS][PITCH]: z_l = (f+ at l, f- at l+1)
@@ -1070,6 +1074,7 @@ template <int DIM, int A, int SCHEME>
 __global__ void __launch_bounds__(THREADS, SCHEME == IBFSA_MLP_TENO5 ? 4 : 5)
     k_conv32_tma(Plan p, const __grid_constant__ CUtensorMap tq,
                  const __grid_constant__ CUtensorMap tw, const __grid_constant__ CUtensorMap tl) {
+  begin_kernel();
   using TT = TmaTile<DIM, A>;
   using T = Tile<A>;
   constexpr int NV = TT::NV, R = TT::R, LEN = TT::LEN, SEG = TT::SEG;
@@ -1295,6 +1300,7 @@ __device__ __forceinline__ void char_term32(const Plan &p, const Free &fs, int a
 // it latency; with one launch the 1021 x 771 wake's six steps went from 2543 to 2143 us.
 template <int DIM>
 __global__ void __launch_bounds__(128) k_char_faces32(Plan p) {
+  begin_kernel();
   constexpr int NV = DIM + 2;
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   int I[3], face = -1;
@@ -1357,6 +1363,7 @@ __global__ void __launch_bounds__(128) k_ib_interp64(Plan p, const double *__res
                                                      const double *__restrict__ xis,
                                                      const double *xin, double *xio, double A,
                                                      double Bc, double dt, int advance) {
+  begin_kernel();
   constexpr int G = marker::Support<DIM>::G;
   const int r = threadIdx.x % G, km = (int)((blockIdx.x * blockDim.x + threadIdx.x) / G);
   const int k = min(km, p.nm - 1);
@@ -1387,6 +1394,7 @@ __global__ void __launch_bounds__(128) k_ib_interp64(Plan p, const double *__res
 template <int DIM>
 __global__ void __launch_bounds__(128) k_spread32(Plan p, const double *__restrict__ Qn,
                                                   const float *__restrict__ din) {
+  begin_kernel();
   constexpr int G = marker::Support<DIM>::G;
   const int r = threadIdx.x % G, km = (int)((blockIdx.x * blockDim.x + threadIdx.x) / G);
   const int k = min(km, p.nm - 1), M = p.max_markers;
@@ -1488,6 +1496,7 @@ __global__ void __launch_bounds__(THREADS) k_finish32(Plan p, const float *__res
                                                       float *__restrict__ dout, double *Qn,
                                                       double *__restrict__ Lout, float Bc,
                                                       float dt, int mode) {
+  begin_kernel();
   constexpr int NV = DIM + 2;
   const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;  // cells fit in 31 bits
   if (t >= (unsigned)p.N) return;
@@ -1521,6 +1530,7 @@ __global__ void __launch_bounds__(THREADS, 4) k_visc_finish32(Plan p, const floa
                                                            float *__restrict__ dout, double *Qn,
                                                            double *__restrict__ Lout, float Bc,
                                                            float dt, int mode) {
+  begin_kernel();
   using namespace v2;
   extern __shared__ float smm[];
   float *su = smm, *sv = su + SX * SY;            // [SY][SX]
@@ -1648,6 +1658,7 @@ __global__ void __launch_bounds__(vm::VT, VM_MIN_BLOCKS) k_visc_march32(Plan p, 
                                                           float *__restrict__ dout, double *Qn,
                                                           double *__restrict__ Lout, float Bc,
                                                           float dt, int mode, int zc) {
+  begin_kernel();
   using namespace vm;
   extern __shared__ float smm[];
   float *ring = smm;                              // [5][3][SY][SX]
@@ -1946,7 +1957,7 @@ cudaError_t launch_conv_x(const Plan &p, int nseg, cudaStream_t st) {
   const long long rows = (long long)p.n[1] * p.n[2];
   const long long blocks = (rows + T::ROWS - 1) / T::ROWS * nseg;
   static_assert(T::BYTES <= 48 * 1024, "within the default dynamic shared memory");
-  k_conv32_x<DIM, SCHEME, LPR><<<(unsigned)blocks, THREADS, T::BYTES, st>>>(p, seg, nseg);
+  launch(k_conv32_x<DIM, SCHEME, LPR>, (unsigned)blocks, THREADS, T::BYTES, st, p, seg, nseg);
   return cudaGetLastError();
 }
 
@@ -1967,7 +1978,7 @@ cudaError_t launch_conv(const Plan &p, int first, cudaStream_t st) {
         int nseg = (p.n[A] + T::SEG - 1) / T::SEG;
         grid = dim3(nseg * ((p.n[0] + T::ROWS - 1) / T::ROWS), A == 1 ? p.n[2] : p.n[1]);
       }
-      k_conv32<DIM, A, SCHEME, true><<<grid, THREADS, smem, st>>>(p, first);
+      launch(k_conv32<DIM, A, SCHEME, true>, grid, THREADS, smem, st, p, first);
       return cudaGetLastError();
     }
   }
@@ -1991,7 +2002,7 @@ cudaError_t launch_conv(const Plan &p, int first, cudaStream_t st) {
       int nseg = (p.n[A] + T::SEG - 1) / T::SEG;
       int nx = (p.n[0] + T::ROWS - 1) / T::ROWS;
       dim3 grid(nseg * nx, A == 1 ? p.n[2] : p.n[1]);
-      k_conv32_tma<DIM, A, SCHEME><<<grid, THREADS, smem, st>>>(p, tq, tw, tl);
+      launch(k_conv32_tma<DIM, A, SCHEME>, grid, THREADS, smem, st, p, tq, tw, tl);
       return cudaGetLastError();
     }
   }
@@ -2009,7 +2020,7 @@ cudaError_t launch_conv(const Plan &p, int first, cudaStream_t st) {
     int nx = (p.n[0] + T::ROWS - 1) / T::ROWS;
     grid = dim3(nseg * nx, A == 1 ? p.n[2] : p.n[1]);
   }
-  k_conv32<DIM, A, SCHEME><<<grid, THREADS, smem, st>>>(p, first);
+  launch(k_conv32<DIM, A, SCHEME>, grid, THREADS, smem, st, p, first);
   return cudaGetLastError();
   }
 }
@@ -2048,14 +2059,14 @@ cudaError_t run_stage(const Plan &p, const StageArgs &s, cudaStream_t st) {
   float *dout = s.stage == 0 ? p.d1 : s.stage == 1 ? p.d2 : nullptr;
   const double *Qn = s.Qn;
   prof_begin(pr, st);
-  k_pad32<DIM><<<blocks_for(p.NP, THREADS), THREADS, 0, st>>>(p, din);
+  launch(k_pad32<DIM>, blocks_for(p.NP, THREADS), THREADS, 0, st, p, din);
   prof_end(pr, K_PAD, st);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   int advance = s.stage >= 0;
   if (p.nm > 0) {
     prof_begin(pr, st);
-    k_ib_interp64<DIM><<<blocks_for((long long)p.nm * marker::Support<DIM>::G, 128), 128, 0, st>>>(
-        p, Qn, din, s.xis, s.xin, s.xio, s.a, s.b, s.dt, advance);
+    launch(k_ib_interp64<DIM>, blocks_for((long long)p.nm * marker::Support<DIM>::G, 128), 128, 0,
+           st, p, Qn, din, s.xis, s.xin, s.xio, s.a, s.b, s.dt, advance);
     prof_end(pr, K_INTERP, st);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
@@ -2076,14 +2087,14 @@ cudaError_t run_stage(const Plan &p, const StageArgs &s, cudaStream_t st) {
   }
   if (const long long cells = char_cells(p)) {
     prof_begin(pr, st);
-    k_char_faces32<DIM><<<blocks_for(cells, 128), 128, 0, st>>>(p);
+    launch(k_char_faces32<DIM>, blocks_for(cells, 128), 128, 0, st, p);
     prof_end(pr, K_CONV_X, st);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   if (p.nm > 0) {
     prof_begin(pr, st);
-    k_spread32<DIM><<<blocks_for((long long)p.nm * marker::Support<DIM>::G, 128), 128, 0, st>>>(
-        p, Qn, din);
+    launch(k_spread32<DIM>, blocks_for((long long)p.nm * marker::Support<DIM>::G, 128), 128, 0, st,
+           p, Qn, din);
     prof_end(pr, K_SPREAD, st);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
@@ -2099,19 +2110,19 @@ cudaError_t run_stage(const Plan &p, const StageArgs &s, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     const int zc = march_chunk(p.n);
     dim3 grid((p.n[0] + TX - 1) / TX, (p.n[1] + TY - 1) / TY, (p.n[2] + zc - 1) / zc);
-    kern<<<grid, VT, SMEM, st>>>(q, din, dout, const_cast<double *>(Qn), s.Lout, (float)s.b,
-                                 (float)s.dt, mode, zc);
+    launch(kern, grid, VT, SMEM, st, q, din, dout, const_cast<double *>(Qn), s.Lout, (float)s.b,
+           (float)s.dt, mode, zc);
   } else if (p.Re > 0.0) {
     using namespace v2;
     const bool stretched = p.minv12_32[0] || p.minv12_32[1];
     auto kern = stretched ? k_visc_finish32<true> : k_visc_finish32<false>;
     static_assert(SMEM <= 48 * 1024, "within the default dynamic shared memory");
     const unsigned tiles = (unsigned)((p.n[0] + TX - 1) / TX) * ((p.n[1] + TY - 1) / TY);
-    kern<<<tiles, THREADS, SMEM, st>>>(q, din, dout, const_cast<double *>(Qn), s.Lout, (float)s.b,
-                                       (float)s.dt, mode);
+    launch(kern, tiles, THREADS, SMEM, st, q, din, dout, const_cast<double *>(Qn), s.Lout,
+           (float)s.b, (float)s.dt, mode);
   } else {
-    k_finish32<DIM><<<blocks_for(p.N, THREADS), THREADS, 0, st>>>(
-        q, din, dout, const_cast<double *>(Qn), s.Lout, (float)s.b, (float)s.dt, mode);
+    launch(k_finish32<DIM>, blocks_for(p.N, THREADS), THREADS, 0, st, q, din, dout,
+           const_cast<double *>(Qn), s.Lout, (float)s.b, (float)s.dt, mode);
   }
   prof_end(pr, K_FINISH, st);
   return cudaGetLastError();
@@ -2318,8 +2329,8 @@ cudaError_t fp32_wavespeed(const Plan &p, const double *Q, cudaStream_t st) {
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(p.alpha_bits, 0, 3 * sizeof(unsigned long long), st);
   if (e != cudaSuccess) return e;
-  if (p.dim == 2) k_pad32<2><<<blocks_for(p.NP, THREADS), THREADS, 0, st>>>(p, nullptr);
-  else k_pad32<3><<<blocks_for(p.NP, THREADS), THREADS, 0, st>>>(p, nullptr);
+  if (p.dim == 2) launch(k_pad32<2>, blocks_for(p.NP, THREADS), THREADS, 0, st, p, nullptr);
+  else launch(k_pad32<3>, blocks_for(p.NP, THREADS), THREADS, 0, st, p, nullptr);
   return cudaGetLastError();
 }
 

@@ -14,6 +14,7 @@
 #include <stdint.h>
 
 #include "ibfsa_internal.h"
+#include "launch.cuh"
 #include "marker.cuh"
 #include "mesh.cuh"
 
@@ -383,6 +384,7 @@ __device__ __forceinline__ double recon(const Plan &p, double a, double b, doubl
 // ------------------------------------------------------------------------------------------
 template <int DIM>
 __global__ void __launch_bounds__(THREADS) k_pad(Plan p, const double *__restrict__ Q) {
+  begin_kernel();
   constexpr int NV = DIM + 2;
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   double wmax[3] = {0.0, 0.0, 0.0};
@@ -596,6 +598,7 @@ __host__ __device__ constexpr size_t conv_smem_bytes() {
 // thread per pass, conservative difference into L
 template <int DIM, int A, int SCHEME>
 __global__ void __launch_bounds__(THREADS) k_conv_char(Plan p, int first) {
+  begin_kernel();
   constexpr int NV = DIM + 2;
   using T = ConvTile<A>;
   extern __shared__ double sm[];
@@ -791,6 +794,7 @@ struct LineTile {
 
 template <int DIM, int A, int SCHEME, int K>
 __global__ void __launch_bounds__(THREADS, 3) k_conv(Plan p, int first, int nseg) {
+  begin_kernel();
   constexpr int NV = DIM + 2;
   using T = LineTile<A, K>;
   // TENO5's weights depend on ratios of indicators only (its floors aside), so its fast form
@@ -979,6 +983,7 @@ __device__ __forceinline__ void char_term(const Plan &p, int a, int side, const 
 // direction, low face first).
 template <int DIM>
 __global__ void __launch_bounds__(128) k_char_faces(Plan p) {
+  begin_kernel();
   constexpr int NV = DIM + 2;
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   int I[3], face = -1;
@@ -1037,6 +1042,7 @@ __device__ __forceinline__ double metric12(const Plan &p, int a, int i, double *
 // 51 operations a cell in 3D instead of 59, 1.98 -> 1.76 ms at 256^3.
 template <int DIM>
 __global__ void __launch_bounds__(THREADS) k_visc_flux(Plan p) {
+  begin_kernel();
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= p.NB) return;
   int bx = (int)(t % p.B[0]);
@@ -1112,6 +1118,7 @@ __global__ void __launch_bounds__(THREADS) k_visc_flux(Plan p) {
 // strict form: the divergence by itself, operation by operation (the fast form's is in k_finish)
 template <int DIM>
 __global__ void __launch_bounds__(THREADS) k_visc_div(Plan p) {
+  begin_kernel();
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= p.N) return;
   int i = (int)(t % p.n[0]);
@@ -1225,6 +1232,7 @@ __device__ __forceinline__ void strict_supports(const Plan &p, int k0,
 template <int DIM>
 __global__ void k_ib_interp(Plan p, const double *__restrict__ xis, const double *xin,
                             double *xio, double A, double Bc, double dt, int advance) {
+  begin_kernel();
   const int nm = p.nm, M = p.max_markers;
   if constexpr (!STRICT) {  // one group of lanes per marker (marker.cuh)
     constexpr int G = marker::Support<DIM>::G;
@@ -1302,6 +1310,7 @@ struct SpreadTable {
 
 template <int DIM>
 __global__ void __launch_bounds__(128) k_spread_table(Plan p, SpreadTable t, int first, int n) {
+  begin_kernel();
   __shared__ double sw[STRICT_MARKERS][3][4], shp[STRICT_MARKERS];
   __shared__ int sj[STRICT_MARKERS][3], sbad[STRICT_MARKERS];
   const int i0 = blockIdx.x * STRICT_MARKERS, tid = threadIdx.x;
@@ -1331,6 +1340,7 @@ struct SpreadTile {
 
 template <int DIM>
 __global__ void __launch_bounds__(THREADS) k_spread_gather(Plan p, SpreadTable t, int first, int n) {
+  begin_kernel();
   using T = SpreadTile<DIM>;
   static_assert(T::X * T::Y * T::Z == THREADS, "one thread per cell");
   __shared__ int list[THREADS], cnt[THREADS / 32];
@@ -1406,9 +1416,10 @@ cudaError_t spread_strict(const Plan &p, cudaStream_t st) {
     t.box = reinterpret_cast<int *>(p.Qp + room);
     cudaError_t e = cudaMemsetAsync(t.box, 0x7f, 6 * sizeof(int), st);
     if (e != cudaSuccess) return e;
-    k_spread_table<DIM><<<(n + STRICT_MARKERS - 1) / STRICT_MARKERS, 128, 0, st>>>(p, t, first, n);
+    launch(k_spread_table<DIM>, (n + STRICT_MARKERS - 1) / STRICT_MARKERS, 128, 0, st, p, t, first,
+           n);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_spread_gather<DIM><<<tiles, THREADS, 0, st>>>(p, t, first, n);
+    launch(k_spread_gather<DIM>, tiles, THREADS, 0, st, p, t, first, n);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -1418,6 +1429,7 @@ cudaError_t spread_strict(const Plan &p, cudaStream_t st) {
 // atomics straight into L: momentum += f, energy += f.u
 template <int DIM>
 __global__ void __launch_bounds__(128) k_spread_atomic(Plan p) {
+  begin_kernel();
   constexpr int G = marker::Support<DIM>::G;
   const int r = threadIdx.x % G, km = (int)((blockIdx.x * blockDim.x + threadIdx.x) / G);
   const int k = min(km, p.nm - 1), M = p.max_markers;
@@ -1458,6 +1470,7 @@ __global__ void __launch_bounds__(THREADS) k_finish(Plan p, const double *__rest
                                                     const double *Qn, double *out, double A,
                                                     double Bc, double dt, int advance,
                                                     ViscScale vs) {
+  begin_kernel();
   constexpr int NV = DIM + 2;
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= p.N) return;
@@ -1586,7 +1599,7 @@ cudaError_t launch_conv_char(const Plan &p, int first, cudaStream_t st) {
     int nx = (p.n[0] + T::ROWS - 1) / T::ROWS;
     grid = dim3(nseg * nx, A == 1 ? p.n[2] : p.n[1]);
   }
-  k_conv_char<DIM, A, SCHEME><<<grid, THREADS, smem, st>>>(p, first);
+  launch(k_conv_char<DIM, A, SCHEME>, grid, THREADS, smem, st, p, first);
   return cudaGetLastError();
 }
 
@@ -1618,7 +1631,7 @@ cudaError_t launch_conv_k(const Plan &p, int first, int nseg, long long tiles, c
   static_assert(smem <= 48 * 1024, "within the default dynamic shared memory");
   static_assert(LineTile<A, K>::FACES <= 32, "the update walks a line of cells with one warp");
   dim3 grid((unsigned)((DIM + 2) * tiles * nseg), A == 2 ? p.n[1] : p.n[2]);
-  k_conv<DIM, A, SCHEME, K><<<grid, THREADS, smem, st>>>(p, first, nseg);
+  launch(k_conv<DIM, A, SCHEME, K>, grid, THREADS, smem, st, p, first, nseg);
   return cudaGetLastError();
 }
 
@@ -1641,7 +1654,7 @@ cudaError_t run_stage(const Plan &p, const StageArgs &s, cudaStream_t st) {
   e = cudaMemsetAsync(p.alpha_bits, 0, 3 * sizeof(unsigned long long), st);
   if (e != cudaSuccess) return e;
   prof_begin(pr, st);
-  k_pad<DIM><<<blocks_for(p.NP, THREADS), THREADS, 0, st>>>(p, s.Qs);
+  launch(k_pad<DIM>, blocks_for(p.NP, THREADS), THREADS, 0, st, p, s.Qs);
   prof_end(pr, K_PAD, st);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   int advance = s.stage >= 0;
@@ -1649,8 +1662,8 @@ cudaError_t run_stage(const Plan &p, const StageArgs &s, cudaStream_t st) {
     prof_begin(pr, st);
     const long long lanes = STRICT ? (p.nm + STRICT_MARKERS - 1LL) / STRICT_MARKERS * 128
                                    : (long long)p.nm * marker::Support<DIM>::G;
-    k_ib_interp<DIM><<<blocks_for(lanes, 128), 128, 0, st>>>(p, s.xis, s.xin, s.xio, s.a, s.b,
-                                                             s.dt, advance);
+    launch(k_ib_interp<DIM>, blocks_for(lanes, 128), 128, 0, st, p, s.xis, s.xin, s.xio, s.a, s.b,
+           s.dt, advance);
     prof_end(pr, K_INTERP, st);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
@@ -1671,7 +1684,7 @@ cudaError_t run_stage(const Plan &p, const StageArgs &s, cudaStream_t st) {
   }
   if (const long long cells = char_cells(p)) {
     prof_begin(pr, st);
-    k_char_faces<DIM><<<blocks_for(cells, 128), 128, 0, st>>>(p);
+    launch(k_char_faces<DIM>, blocks_for(cells, 128), 128, 0, st, p);
     prof_end(pr, K_CONV_X, st);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
@@ -1684,8 +1697,8 @@ cudaError_t run_stage(const Plan &p, const StageArgs &s, cudaStream_t st) {
     if constexpr (STRICT) {
       es = spread_strict<DIM>(p, st);
     } else {
-      k_spread_atomic<DIM><<<blocks_for((long long)p.nm * marker::Support<DIM>::G, 128), 128, 0,
-                             st>>>(p);
+      launch(k_spread_atomic<DIM>, blocks_for((long long)p.nm * marker::Support<DIM>::G, 128), 128,
+             0, st, p);
       es = cudaGetLastError();
     }
     prof_end(pr, K_SPREAD, st);
@@ -1696,14 +1709,14 @@ cudaError_t run_stage(const Plan &p, const StageArgs &s, cudaStream_t st) {
   const bool viscous = p.Re > 0.0;
   if (viscous) {
     prof_begin(pr, st);
-    k_visc_flux<DIM><<<blocks_for(p.NB, THREADS), THREADS, 0, st>>>(p);
+    launch(k_visc_flux<DIM>, blocks_for(p.NB, THREADS), THREADS, 0, st, p);
     prof_end(pr, K_VISC_FLUX, st);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   if constexpr (STRICT) {
     if (viscous) {
       prof_begin(pr, st);
-      k_visc_div<DIM><<<blocks_for(p.N, THREADS), THREADS, 0, st>>>(p);
+      launch(k_visc_div<DIM>, blocks_for(p.N, THREADS), THREADS, 0, st, p);
       prof_end(pr, K_VISC_DIV, st);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
@@ -1717,11 +1730,11 @@ cudaError_t run_stage(const Plan &p, const StageArgs &s, cudaStream_t st) {
   for (int a = 0; a < DIM; a++) vs.c[a] = p.mm[a] ? p.inv_Re : p.inv_h12[a] * p.inv_Re;
   const unsigned blocks = blocks_for(p.N, THREADS);
   if (!STRICT && viscous)
-    k_finish<DIM, !STRICT><<<blocks, THREADS, 0, st>>>(q, s.Qs, s.Qn, out, s.a, s.b, s.dt, advance,
-                                                      vs);
+    launch(k_finish<DIM, !STRICT>, blocks, THREADS, 0, st, q, s.Qs, s.Qn, out, s.a, s.b, s.dt,
+           advance, vs);
   else
-    k_finish<DIM, false><<<blocks, THREADS, 0, st>>>(q, s.Qs, s.Qn, out, s.a, s.b, s.dt, advance,
-                                                    vs);
+    launch(k_finish<DIM, false>, blocks, THREADS, 0, st, q, s.Qs, s.Qn, out, s.a, s.b, s.dt,
+           advance, vs);
   prof_end(pr, K_FINISH, st);
   return cudaGetLastError();
 }
@@ -1737,8 +1750,8 @@ inline cudaError_t stage_impl(const Plan &p, const StageArgs &s, cudaStream_t st
 inline cudaError_t wavespeed_impl(const Plan &p, const double *Q, cudaStream_t st) {
   cudaError_t e = cudaMemsetAsync(p.alpha_bits, 0, 3 * sizeof(unsigned long long), st);
   if (e != cudaSuccess) return e;
-  if (p.dim == 2) k_pad<2><<<blocks_for(p.NP, THREADS), THREADS, 0, st>>>(p, Q);
-  else k_pad<3><<<blocks_for(p.NP, THREADS), THREADS, 0, st>>>(p, Q);
+  if (p.dim == 2) launch(k_pad<2>, blocks_for(p.NP, THREADS), THREADS, 0, st, p, Q);
+  else launch(k_pad<3>, blocks_for(p.NP, THREADS), THREADS, 0, st, p, Q);
   return cudaGetLastError();
 }
 
