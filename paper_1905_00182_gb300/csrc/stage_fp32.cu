@@ -1356,58 +1356,56 @@ __device__ __forceinline__ double stage_q(const Plan &p, const double *__restric
   return din ? v + (double)din[c * p.N + o] : v;
 }
 
-// Interpolation (Eq. 8) and penalty force (Eq. 7), one group of lanes per marker (marker.cuh).
-template <int DIM>
-__global__ void __launch_bounds__(128) k_ib_interp64(Plan p, const double *__restrict__ Qn,
-                                                     const float *__restrict__ din,
-                                                     const double *__restrict__ xis,
-                                                     const double *xin, double *xio, double A,
-                                                     double Bc, double dt, int advance) {
+// Markers, a group of G lanes each (marker.cuh).  Interpolation (Eq. 8) and penalty force (Eq. 7) in
+// FP64, and the spreading (Eq. 9) into the FP32 right-hand side: the kernel weights and the
+// marker's force are FP64; the per-cell force, the fluid velocity of the power term f.u and the
+// atomic additions are FP32, the precision of the right-hand side they enter.
+template <int DIM, int G, int PART>
+__global__ void __launch_bounds__(128) k_markers32(Plan p, const double *__restrict__ Qn,
+                                                   const float *__restrict__ din,
+                                                   const double *__restrict__ xis,
+                                                   const double *xin, double *xio, double A,
+                                                   double Bc, double dt, int advance) {
   begin_kernel();
-  constexpr int G = marker::Support<DIM>::G;
-  const int r = threadIdx.x % G, km = (int)((blockIdx.x * blockDim.x + threadIdx.x) / G);
-  const int k = min(km, p.nm - 1);
-  const marker::Support<DIM> t = marker::support<DIM>(p, p.X, p.max_markers, k, r);
-  double acc[DIM];
-#pragma unroll
-  for (int a = 0; a < DIM; a++) acc[a] = 0.0;
-  if (t.ok) {
-    const long long o = int_index(p, t.j0[0], t.j0[1] + (r & 3), t.j0[2] + (r >> 2));
-#pragma unroll
-    for (int r0 = 0; r0 < 4; r0++) {
-      const double wi = t.w0[r0] * (1.0 / stage_q(p, Qn, din, 0, o + r0));
-#pragma unroll
-      for (int a = 0; a < DIM; a++) acc[a] = fma(stage_q(p, Qn, din, 1 + a, o + r0), wi, acc[a]);
-    }
-  }
-#pragma unroll
-  for (int a = 0; a < DIM; a++) acc[a] = marker::group_sum<DIM>(acc[a] * t.wr);
-  if (km >= p.nm) return;
-  if (t.ok) marker::force<DIM>(p, k, r, acc, xis, xin, xio, A, Bc, dt, advance);
-  else marker::off_grid<DIM>(p, k, r, xin, xio, advance);
-}
-
-// Spreading (Eq. 9) into the FP32 right-hand side, one group of lanes per marker (marker.cuh),
-// four support cells per lane.  The kernel weights and the marker's force are FP64; the per-cell
-// force, the fluid velocity of the power term f.u and the atomic additions are FP32, the
-// precision of the right-hand side they enter.
-template <int DIM>
-__global__ void __launch_bounds__(128) k_spread32(Plan p, const double *__restrict__ Qn,
-                                                  const float *__restrict__ din) {
-  begin_kernel();
-  constexpr int G = marker::Support<DIM>::G;
+  constexpr int C = marker::Support<DIM, G>::C;
   const int r = threadIdx.x % G, km = (int)((blockIdx.x * blockDim.x + threadIdx.x) / G);
   const int k = min(km, p.nm - 1), M = p.max_markers;
-  const marker::Support<DIM> t = marker::support<DIM>(p, p.X, M, k, r);
-  if (km >= p.nm || !t.ok) return;  // the interpolation kernel reports markers off the grid
+  const auto t = marker::support<DIM, G>(p, p.X, M, k, r);
+  const long long o = int_index(p, t.c0[0], t.c0[1], t.c0[2]);
+  double F[DIM];
+  if constexpr (PART & marker::INTERP) {
+    double acc[DIM];
+#pragma unroll
+    for (int a = 0; a < DIM; a++) acc[a] = 0.0;
+    if (t.ok) {
+#pragma unroll
+      for (int r0 = 0; r0 < C; r0++) {
+        const double wi = t.w0[r0] * (1.0 / stage_q(p, Qn, din, 0, o + r0));
+#pragma unroll
+        for (int a = 0; a < DIM; a++)
+          acc[a] = fma(stage_q(p, Qn, din, 1 + a, o + r0), wi, acc[a]);
+      }
+    }
+#pragma unroll
+    for (int a = 0; a < DIM; a++) acc[a] = marker::group_sum<G>(acc[a] * t.wr);
+    double mine = 0.0;
+    if (km < p.nm) {
+      if (t.ok) mine = marker::force<DIM>(p, k, r, acc, xis, xin, xio, A, Bc, dt, advance);
+      else marker::off_grid<DIM>(p, k, r, xin, xio, advance);
+    }
+#pragma unroll
+    for (int a = 0; a < DIM; a++) F[a] = __shfl_sync(0xffffffffu, mine, a, G);
+  }
+  if constexpr (!(PART & marker::SPREAD)) return;
+  if (km >= p.nm || !t.ok) return;  // the interpolation reports markers off the grid
   const double sc = p.dS[k] * t.ihp;
   float f[DIM];
 #pragma unroll
-  for (int a = 0; a < DIM; a++) f[a] = (float)(-p.F[a * M + k] * sc);
+  for (int a = 0; a < DIM; a++)
+    f[a] = (float)(-(PART & marker::INTERP ? F[a] : p.F[a * M + k]) * sc);
   const Free fs = free_stream(p);
-  const long long o = int_index(p, t.j0[0], t.j0[1] + (r & 3), t.j0[2] + (r >> 2));
 #pragma unroll
-  for (int r0 = 0; r0 < 4; r0++) {
+  for (int r0 = 0; r0 < C; r0++) {
     const float wt = (float)(t.w0[r0] * t.wr);
     const float d0 = p.qn32[o + r0] + (din ? din[o + r0] : 0.f);
     const float inv_rho = 1.f / (fs.rho + d0);
@@ -2063,13 +2061,22 @@ cudaError_t run_stage(const Plan &p, const StageArgs &s, cudaStream_t st) {
   prof_end(pr, K_PAD, st);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   int advance = s.stage >= 0;
-  if (p.nm > 0) {
+  auto markers = [&](auto part, int cls) -> cudaError_t {
+    if (p.nm <= 0) return cudaSuccess;
     prof_begin(pr, st);
-    launch(k_ib_interp64<DIM>, blocks_for((long long)p.nm * marker::Support<DIM>::G, 128), 128, 0,
-           st, p, Qn, din, s.xis, s.xin, s.xio, s.a, s.b, s.dt, advance);
-    prof_end(pr, K_INTERP, st);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
+    marker::with_group<DIM>(p.nm, [&](auto g) {
+      launch(k_markers32<DIM, g(), part()>, blocks_for((long long)p.nm * g(), 128), 128, 0, st, p,
+             Qn, din, s.xis, s.xin, s.xio, s.a, s.b, s.dt, advance);
+    });
+    prof_end(pr, cls, st);
+    return cudaGetLastError();
+  };
+  // interpolation and spreading in one launch after the convective term, unless someone waits for
+  // the forces
+  using Interp = std::integral_constant<int, marker::INTERP>;
+  using Spread = std::integral_constant<int, marker::SPREAD>;
+  using Both = std::integral_constant<int, marker::BOTH>;
+  if (s.forces && (e = markers(Interp(), K_INTERP)) != cudaSuccess) return e;
   if (s.forces && (e = cudaEventRecord(s.forces, st)) != cudaSuccess) return e;
   prof_begin(pr, st);
   e = launch_conv<DIM, 0, SCHEME>(p, 1, st);
@@ -2091,13 +2098,8 @@ cudaError_t run_stage(const Plan &p, const StageArgs &s, cudaStream_t st) {
     prof_end(pr, K_CONV_X, st);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  if (p.nm > 0) {
-    prof_begin(pr, st);
-    launch(k_spread32<DIM>, blocks_for((long long)p.nm * marker::Support<DIM>::G, 128), 128, 0, st,
-           p, Qn, din);
-    prof_end(pr, K_SPREAD, st);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
+  e = s.forces ? markers(Spread(), K_SPREAD) : markers(Both(), K_SPREAD);
+  if (e != cudaSuccess) return e;
   int mode = !advance ? 0 : (s.stage < 2 ? 1 : 2);
   Plan q = p;
   q.src_scale = s.src_scale;

@@ -1227,67 +1227,45 @@ __device__ __forceinline__ void strict_supports(const Plan &p, int k0,
   }
 }
 
-// U_ib = sum_j u_j prod lambda (Eq. 8), F = alpha xi + beta (U_ib - U) (Eq. 7), and the RK
-// update of xi (xi' = U_ib - U) when the stage is advanced
+// strict form: U_ib = sum_j u_j prod lambda (Eq. 8), F = alpha xi + beta (U_ib - U) (Eq. 7), and the
+// RK update of xi (xi' = U_ib - U) when the stage is advanced
 template <int DIM>
 __global__ void k_ib_interp(Plan p, const double *__restrict__ xis, const double *xin,
                             double *xio, double A, double Bc, double dt, int advance) {
   begin_kernel();
   const int nm = p.nm, M = p.max_markers;
-  if constexpr (!STRICT) {  // one group of lanes per marker (marker.cuh)
-    constexpr int G = marker::Support<DIM>::G;
-    const int r = threadIdx.x % G, km = (int)((blockIdx.x * blockDim.x + threadIdx.x) / G);
-    const int k = min(km, nm - 1);
-    const marker::Support<DIM> t = marker::support<DIM>(p, p.X, M, k, r);
-    double acc[DIM];
+  // strict: the weights of SM markers one per thread, the products u (w w w) of their support
+  // cells one per thread, then one thread per marker and component adds them up in the order of
+  // the formula (z, y, x)
+  constexpr int S = strict_support_cells<DIM>, SM = STRICT_MARKERS;
+  __shared__ double sw[SM][3][4], sv[SM][DIM][S + 1];
+  __shared__ int sj[SM][3], sbad[SM];
+  const int k0 = blockIdx.x * SM, tid = threadIdx.x;
+  strict_supports<DIM>(p, k0, sw, sj, sbad, nullptr);
+  for (int e = tid; e < SM * S; e += blockDim.x) {
+    const int m = e / S, r = e % S, r0 = r & 3, r1 = (r >> 2) & 3, r2 = r >> 4;
+    if (k0 + m >= nm || sbad[m]) continue;
+    const double wt = sw[m][0][r0] * sw[m][1][r1] * sw[m][2][r2];
+    const long long o = pad_index(p, sj[m][0] + r0, sj[m][1] + r1, sj[m][2] + r2);
 #pragma unroll
-    for (int a = 0; a < DIM; a++) acc[a] = 0.0;
-    if (t.ok) {
-      const long long s = pad_index(p, t.j0[0], t.j0[1] + (r & 3), t.j0[2] + (r >> 2));
-#pragma unroll
-      for (int a = 0; a < DIM; a++)
-#pragma unroll
-        for (int r0 = 0; r0 < 4; r0++) acc[a] = fma(p.Wp[a * p.NP + s + r0], t.w0[r0], acc[a]);
+    for (int a = 0; a < DIM; a++) sv[m][a][r] = p.Wp[a * p.NP + o] * wt;
+  }
+  __syncthreads();
+  for (int e = tid; e < SM * DIM; e += blockDim.x) {
+    const int m = e / DIM, a = e % DIM, k = k0 + m;
+    if (k >= nm) continue;
+    if (sbad[m]) {
+      if (a == 0) atomicOr(p.status, IBFSA_STATUS_BOUNDS);
+      p.F[a * M + k] = 0.0;
+      if (advance) xio[a * M + k] = xin[a * M + k];
+      continue;
     }
-#pragma unroll
-    for (int a = 0; a < DIM; a++) acc[a] = marker::group_sum<DIM>(acc[a] * t.wr);
-    if (km >= nm) return;
-    if (t.ok) marker::force<DIM>(p, k, r, acc, xis, xin, xio, A, Bc, dt, advance);
-    else marker::off_grid<DIM>(p, k, r, xin, xio, advance);
-  } else {
-    // strict: the weights of SM markers one per thread, the products u (w w w) of their support
-    // cells one per thread, then one thread per marker and component adds them up in the order of
-    // the formula (z, y, x)
-    constexpr int S = strict_support_cells<DIM>, SM = STRICT_MARKERS;
-    __shared__ double sw[SM][3][4], sv[SM][DIM][S + 1];
-    __shared__ int sj[SM][3], sbad[SM];
-    const int k0 = blockIdx.x * SM, tid = threadIdx.x;
-    strict_supports<DIM>(p, k0, sw, sj, sbad, nullptr);
-    for (int e = tid; e < SM * S; e += blockDim.x) {
-      const int m = e / S, r = e % S, r0 = r & 3, r1 = (r >> 2) & 3, r2 = r >> 4;
-      if (k0 + m >= nm || sbad[m]) continue;
-      const double wt = sw[m][0][r0] * sw[m][1][r1] * sw[m][2][r2];
-      const long long o = pad_index(p, sj[m][0] + r0, sj[m][1] + r1, sj[m][2] + r2);
-#pragma unroll
-      for (int a = 0; a < DIM; a++) sv[m][a][r] = p.Wp[a * p.NP + o] * wt;
-    }
-    __syncthreads();
-    for (int e = tid; e < SM * DIM; e += blockDim.x) {
-      const int m = e / DIM, a = e % DIM, k = k0 + m;
-      if (k >= nm) continue;
-      if (sbad[m]) {
-        if (a == 0) atomicOr(p.status, IBFSA_STATUS_BOUNDS);
-        p.F[a * M + k] = 0.0;
-        if (advance) xio[a * M + k] = xin[a * M + k];
-        continue;
-      }
-      double acc = 0.0;
+    double acc = 0.0;
 #pragma unroll 8
-      for (int r = 0; r < S; r++) acc += sv[m][a][r];
-      double slip = acc - p.U[a * M + k];
-      p.F[a * M + k] = p.alpha_pen * xis[a * M + k] + p.beta_pen * slip;
-      if (advance) xio[a * M + k] = A * xin[a * M + k] + Bc * (xis[a * M + k] + dt * slip);
-    }
+    for (int r = 0; r < S; r++) acc += sv[m][a][r];
+    double slip = acc - p.U[a * M + k];
+    p.F[a * M + k] = p.alpha_pen * xis[a * M + k] + p.beta_pen * slip;
+    if (advance) xio[a * M + k] = A * xin[a * M + k] + Bc * (xis[a * M + k] + dt * slip);
   }
 }
 
@@ -1425,24 +1403,48 @@ cudaError_t spread_strict(const Plan &p, cudaStream_t st) {
   return cudaSuccess;
 }
 
-// fast spreading: one group of lanes per marker, four support cells per lane (marker.cuh),
-// atomics straight into L: momentum += f, energy += f.u
-template <int DIM>
-__global__ void __launch_bounds__(128) k_spread_atomic(Plan p) {
+// Fast form: markers, a group of G lanes each (marker.cuh): interpolation and penalty force, and the
+// spreading with atomics straight into L: momentum += f, energy += f.u
+template <int DIM, int G, int PART>
+__global__ void __launch_bounds__(128) k_markers(Plan p, const double *__restrict__ xis,
+                                                 const double *xin, double *xio, double A,
+                                                 double Bc, double dt, int advance) {
   begin_kernel();
-  constexpr int G = marker::Support<DIM>::G;
+  constexpr int C = marker::Support<DIM, G>::C;
   const int r = threadIdx.x % G, km = (int)((blockIdx.x * blockDim.x + threadIdx.x) / G);
   const int k = min(km, p.nm - 1), M = p.max_markers;
-  const marker::Support<DIM> t = marker::support<DIM>(p, p.X, M, k, r);
+  const auto t = marker::support<DIM, G>(p, p.X, M, k, r);
+  const long long s = pad_index(p, t.c0[0], t.c0[1], t.c0[2]);
+  double F[DIM];
+  if constexpr (PART & marker::INTERP) {
+    double acc[DIM];
+#pragma unroll
+    for (int a = 0; a < DIM; a++) acc[a] = 0.0;
+    if (t.ok) {
+#pragma unroll
+      for (int a = 0; a < DIM; a++)
+#pragma unroll
+        for (int r0 = 0; r0 < C; r0++) acc[a] = fma(p.Wp[a * p.NP + s + r0], t.w0[r0], acc[a]);
+    }
+#pragma unroll
+    for (int a = 0; a < DIM; a++) acc[a] = marker::group_sum<G>(acc[a] * t.wr);
+    double mine = 0.0;
+    if (km < p.nm) {
+      if (t.ok) mine = marker::force<DIM>(p, k, r, acc, xis, xin, xio, A, Bc, dt, advance);
+      else marker::off_grid<DIM>(p, k, r, xin, xio, advance);
+    }
+#pragma unroll
+    for (int a = 0; a < DIM; a++) F[a] = __shfl_sync(0xffffffffu, mine, a, G);
+  }
+  if constexpr (!(PART & marker::SPREAD)) return;
   if (km >= p.nm || !t.ok) return;
-  const long long o = int_index(p, t.j0[0], t.j0[1] + (r & 3), t.j0[2] + (r >> 2));
-  const long long s = pad_index(p, t.j0[0], t.j0[1] + (r & 3), t.j0[2] + (r >> 2));
+  const long long o = int_index(p, t.c0[0], t.c0[1], t.c0[2]);
   const double sc = t.wr * (p.dS[k] * t.ihp);
   double f[DIM];
 #pragma unroll
-  for (int a = 0; a < DIM; a++) f[a] = -p.F[a * M + k] * sc;
+  for (int a = 0; a < DIM; a++) f[a] = -(PART & marker::INTERP ? F[a] : p.F[a * M + k]) * sc;
 #pragma unroll
-  for (int r0 = 0; r0 < 4; r0++) {
+  for (int r0 = 0; r0 < C; r0++) {
     double pw = 0.0;
 #pragma unroll
     for (int a = 0; a < DIM; a++) {
@@ -1658,15 +1660,30 @@ cudaError_t run_stage(const Plan &p, const StageArgs &s, cudaStream_t st) {
   prof_end(pr, K_PAD, st);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   int advance = s.stage >= 0;
-  if (p.nm > 0) {
+  // Markers.  Strict: interpolation now, spreading after the viscous term.  Fast: both in one launch
+  // after the convective term, unless someone waits for the forces.
+  using Interp = std::integral_constant<int, marker::INTERP>;
+  using Spread = std::integral_constant<int, marker::SPREAD>;
+  using Both = std::integral_constant<int, marker::BOTH>;
+  auto markers = [&](auto part) -> cudaError_t {
+    if (p.nm <= 0) return cudaSuccess;
+    cudaError_t es = cudaSuccess;
     prof_begin(pr, st);
-    const long long lanes = STRICT ? (p.nm + STRICT_MARKERS - 1LL) / STRICT_MARKERS * 128
-                                   : (long long)p.nm * marker::Support<DIM>::G;
-    launch(k_ib_interp<DIM>, blocks_for(lanes, 128), 128, 0, st, p, s.xis, s.xin, s.xio, s.a, s.b,
-           s.dt, advance);
-    prof_end(pr, K_INTERP, st);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
+    if constexpr (!STRICT) {
+      marker::with_group<DIM>(p.nm, [&](auto g) {
+        launch(k_markers<DIM, g(), part()>, blocks_for((long long)p.nm * g(), 128), 128, 0, st, p,
+               s.xis, s.xin, s.xio, s.a, s.b, s.dt, advance);
+      });
+    } else if constexpr (part() == marker::INTERP) {
+      launch(k_ib_interp<DIM>, (p.nm + STRICT_MARKERS - 1) / STRICT_MARKERS, 128, 0, st, p, s.xis,
+             s.xin, s.xio, s.a, s.b, s.dt, advance);
+    } else {
+      es = spread_strict<DIM>(p, st);
+    }
+    prof_end(pr, part() == marker::INTERP ? K_INTERP : K_SPREAD, st);
+    return es != cudaSuccess ? es : cudaGetLastError();
+  };
+  if ((STRICT || s.forces) && (e = markers(Interp())) != cudaSuccess) return e;
   if (s.forces && (e = cudaEventRecord(s.forces, st)) != cudaSuccess) return e;
   prof_begin(pr, st);
   e = launch_conv<DIM, 0, SCHEME>(p, 1, st);
@@ -1690,22 +1707,10 @@ cudaError_t run_stage(const Plan &p, const StageArgs &s, cudaStream_t st) {
   }
   // strict: the viscous divergence into L, then the spreading; fast: the spreading, then the
   // divergence as part of finish
-  auto spread = [&]() -> cudaError_t {
-    if (p.nm <= 0) return cudaSuccess;
-    prof_begin(pr, st);
-    cudaError_t es;
-    if constexpr (STRICT) {
-      es = spread_strict<DIM>(p, st);
-    } else {
-      launch(k_spread_atomic<DIM>, blocks_for((long long)p.nm * marker::Support<DIM>::G, 128), 128,
-             0, st, p);
-      es = cudaGetLastError();
-    }
-    prof_end(pr, K_SPREAD, st);
-    return es;
-  };
-  if constexpr (!STRICT)
-    if ((e = spread()) != cudaSuccess) return e;
+  if constexpr (!STRICT) {
+    e = s.forces ? markers(Spread()) : markers(Both());
+    if (e != cudaSuccess) return e;
+  }
   const bool viscous = p.Re > 0.0;
   if (viscous) {
     prof_begin(pr, st);
@@ -1720,7 +1725,7 @@ cudaError_t run_stage(const Plan &p, const StageArgs &s, cudaStream_t st) {
       prof_end(pr, K_VISC_DIV, st);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    if ((e = spread()) != cudaSuccess) return e;
+    if ((e = markers(Spread())) != cudaSuccess) return e;
   }
   double *out = advance ? s.Qo : s.Lout;
   prof_begin(pr, st);
