@@ -1440,6 +1440,37 @@ __device__ __forceinline__ float pressure_source32(const Plan &p, int dim, int i
   return expf(-(float)(p.src_b * 0.693147180559945309417) * r2) * (float)p.src_scale;
 }
 
+// (double)x and (float)x (to nearest, ties to even) by integer operations and, for subnormal x, one
+// FP32 product: a conversion instruction issues at the FP64 rate, 1.8 lanes per clock and SM, so the
+// two conversions and two additions per component of the FP64 update made the last stage FP64-bound.
+// Subnormal values are common (products of small perturbations), so no case is left to the
+// instruction: it would be issued for the whole warp.
+__device__ __forceinline__ double widen(float x) {
+  const bool sub = (__float_as_uint(x) << 1) < (1u << 24);
+  const unsigned b = __float_as_uint(sub ? x * 16777216.f : x), m = b << 1;
+  const unsigned bias = sub ? 896u - 24u : m >= (255u << 24) ? 2u * 896u : 896u;
+  const unsigned hi = m ? (m >> 4) + (bias << 20) : 0u;
+  return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(b << 29));
+}
+
+__device__ __forceinline__ float narrow(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned m = hi & 0x7fffffffu, e = m >> 20;
+  // the result's bits before rounding and what follows them; a carry runs into the exponent
+  unsigned f = __funnelshift_l(lo, m - (896u << 20), 3), rest = lo << 3;
+  if (e < 897u) {  // subnormal or zero
+    const unsigned full = 0x800000u | (f & 0x7fffffu), shift = 897u - e;
+    const bool some = shift <= 24u;
+    f = some ? full >> shift : 0u;
+    rest = some ? full << (32u - shift) | (rest != 0u) : 0u;
+  } else if (e > 1150u) {  // too large, infinite or not a number
+    f = m > 0x7ff00000u || (m == 0x7ff00000u && lo) ? 0x7fffffffu : 0x7f800000u;
+    rest = 0u;
+  }
+  const unsigned up = rest > 0x80000000u || (rest == 0x80000000u && (f & 1u));
+  return __uint_as_float((f + up) | (hi & 0x80000000u));
+}
+
 // The end of a stage at one cell: sponge and pressure source on the right-hand side Lc of cell
 // (i, j, k), offset t, stage increment Dc, then the right-hand side out (mode 0) or the RK update
 template <int DIM, bool STRETCHED>
@@ -1464,7 +1495,7 @@ __device__ __forceinline__ void finish_cell(const Plan &p, float (&Lc)[DIM + 2],
   if (p.src_on) Lc[NV - 1] += pressure_source32<STRETCHED>(p, DIM, i, j, k);
   if (mode == 0) {
 #pragma unroll
-    for (int c = 0; c < NV; c++) Lout[c * p.N + t] = (double)Lc[c];
+    for (int c = 0; c < NV; c++) Lout[c * p.N + t] = widen(Lc[c]);
     return;
   }
   bool bad = false;
@@ -1478,11 +1509,20 @@ __device__ __forceinline__ void finish_cell(const Plan &p, float (&Lc)[DIM + 2],
 #pragma unroll
     for (int c = 0; c < NV; c++) dout[c * p.N + t] = inc[c];
   } else {
+    // The compiler has to take every store for one to Qn, so loads come one after the other unless
+    // they stand before the first store: last stage at 2048^2 126 -> 104 us (152 with conversion
+    // instructions).  Not in 3D, where the march has no registers for them (909 instead of 691 us at
+    // 256^3; 788 with conversion instructions).
+    constexpr bool AHEAD = DIM == 2;
+    double q[NV];
+#pragma unroll
+    for (int c = 0; c < NV; c++)
+      if (AHEAD) q[c] = Qn[c * p.N + t];
 #pragma unroll
     for (int c = 0; c < NV; c++) {
-      double q = Qn[c * p.N + t] + (double)inc[c];
-      Qn[c * p.N + t] = q;
-      p.qn32[c * p.N + t] = (float)(q - p.qinf[c]);
+      q[c] = (AHEAD ? q[c] : Qn[c * p.N + t]) + widen(inc[c]);
+      Qn[c * p.N + t] = q[c];
+      p.qn32[c * p.N + t] = narrow(q[c] - p.qinf[c]);
     }
   }
   if (bad) atomicOr(p.status, IBFSA_STATUS_NONFINITE);
