@@ -1560,7 +1560,8 @@ __global__ void __launch_bounds__(THREADS) k_finish32(Plan p, const float *__res
 // and RK update.  The right-hand side and the stage increment are loaded while the fluxes are
 // evaluated.  Before, a kernel wrote the six flux arrays and the finish pass read them (48 B of
 // 136 per cell and stage) and both found their cell by 64-bit divisions:
-// together 132 -> 85 us per stage at 2048^2 and 244 -> 157 us at 4096 x 2048 (event times).
+// together 132 -> 85 us per stage at 2048^2 and 244 -> 157 us at 4096 x 2048 (event times); 69 and
+// 125 us with the update of finish_cell as it is now, of which the last stage takes half.
 namespace v2 {
 constexpr int TX = 64, TY = 16, PER = TX * TY / THREADS;  // cells of a block, per thread
 constexpr int SX = TX + 8, SY = TY + 8;                   // staged points
@@ -1929,12 +1930,14 @@ __global__ void __launch_bounds__(vm::VT, VM_MIN_BLOCKS) k_visc_march32(Plan p, 
   }
 }
 
+// the rounded state of a new FP64 state, bound by the FP64 pipe (hence narrow): once per state set,
+// 512^3 and two steps 69.1 -> 68.4 ms, 4096 x 2048 and two coupled steps 2.86 -> 2.83
 template <int DIM>
 __global__ void __launch_bounds__(THREADS) k_refresh32(Plan p, const double *__restrict__ Q) {
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= p.N) return;
 #pragma unroll
-  for (int c = 0; c < DIM + 2; c++) p.qn32[c * p.N + t] = (float)(Q[c * p.N + t] - p.qinf[c]);
+  for (int c = 0; c < DIM + 2; c++) p.qn32[c * p.N + t] = narrow(Q[c * p.N + t] - p.qinf[c]);
 }
 
 template <int DIM>
@@ -2073,7 +2076,8 @@ cudaError_t launch_conv(const Plan &p, int first, cudaStream_t st) {
 // pass is bound by latency per plane), so the chunk that minimises (waves of 152 SMs x 4 blocks)
 // x (zc + 7) is taken: long chunks where the columns alone fill the chip, short ones where they
 // do not.  Against a fixed chunk of 64: 99 x 77 x 85 (80 blocks, now 600) 160 -> 45 us, 128^3
-// 176 -> 86 us, 512^3 (chunk 128) 3.80 -> 3.76 ms.
+// 176 -> 86 us, 512^3 (chunk 128) 3.80 -> 3.76 ms (the whole pass since: 42, 79 us and
+// 3.25 ms).
 inline int march_chunk(const int n[3]) {
   const long long cols =
       (long long)((n[0] + vm::TX - 1) / vm::TX) * ((n[1] + vm::TY - 1) / vm::TY);

@@ -7,6 +7,8 @@
 // Per stage:  pad (ghosts + primitives + split speeds)  ->  IB interpolation and penalty force
 //   (Eq. 7-8)  ->  convective flux differences x, y, z  ->  viscous fluxes and their divergence
 //   (Eq. 2-5)  ->  IB spreading (Eq. 9)  ->  finish (sponge, IB source, RK combination).
+// The fast form interpolates and spreads in one kernel between the convective and the viscous terms
+// (unless the caller waits for the forces) and takes the viscous divergence in finish.
 #pragma once
 
 #include <cuda_runtime.h>
