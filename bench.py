@@ -651,8 +651,11 @@ def run_ours(args, rank, world, local_rank):
 
     peaks, peak_kind = measured_peaks()
     fl = flops_per_cell(args.scheme)
-    fl["finish"] = fl["finish"] + (fl["visc_div"] if fp32 else 0)  # FP32 finish fuses the divergence
+    fl["finish"] = fl["finish"] + fl["visc_div"]  # the update kernel takes the viscous divergence
     by = bytes_per_cell(args.precision)
+    if not fp32:  # the symmetric viscous stress is stored once: 9 flux arrays, read by the update
+        by["visc_flux"] = 8 * 3 + 8 * 9
+        by["finish"] += 8 * 9
     sm_mhz = clk["sm_mhz"] or 2070.0
     if fp32:
         peak_tf = FP32_FLOP_PER_CLK_PER_SM * SMS * sm_mhz * 1e6 / 1e12
