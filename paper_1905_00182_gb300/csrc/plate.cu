@@ -999,6 +999,17 @@ int ibfsa_fsi_step(ibfsa_grid *g, ibfsa_plate *p, double dt, int nsteps) {
   // 2.47 -> 2.06 ms; 4096 x 2048 in FP32, 40 elements: two steps 3.97 -> 3.71 ms.  With kernel
   // timing on, everything stays on the grid's stream.
   const bool aside = !G.prof.on;
+  bool forked = false;  // work on the side stream that the grid's does not wait for yet
+  // Has the grid's stream wait for the side stream; before every return, as the caller orders what
+  // comes next (and ends a capture) by the grid's stream alone.  Returns the first error.
+  auto join = [&](cudaError_t first) {
+    if (!forked) return first;
+    forked = false;
+    cudaError_t e = cudaEventRecord(P.moved, P.side);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(G.stream, P.moved, 0);
+    if (e != cudaSuccess) cudaStreamSynchronize(P.side);
+    return first != cudaSuccess ? first : e;
+  };
   for (int step = 0; step < nsteps; step++) {
     prof_begin(&G.prof, G.stream);
     plate::k_markers<<<(nm + 127) / 128, 128, 0, G.stream>>>(P.P, P.e, P.v, P.mk_el, P.mk_S,
@@ -1031,18 +1042,15 @@ int ibfsa_fsi_step(ibfsa_grid *g, ibfsa_plate *p, double dt, int nsteps) {
       const cudaStream_t st = a.forces ? P.side : G.stream;
       if (a.forces) e = cudaStreamWaitEvent(st, P.forces, 0);
       if (e != cudaSuccess) return cuda_err(e, "ibfsa_fsi_step forces");
+      forked = a.forces != nullptr;
       prof_begin(&G.prof, st);
       plate::k_force_average<<<(2 * nm + 127) / 128, 128, 0, st>>>(nm, G.p.F, M, P.Fbar, Wt[s],
                                                                     s == 0);
       prof_end(&G.prof, K_PLATE, st);
       e = cudaGetLastError();
-      if (e != cudaSuccess) return cuda_err(e, "ibfsa_fsi_step force average");
+      if (e != cudaSuccess) return cuda_err(join(e), "ibfsa_fsi_step force average");
     }
-    e = launch_step(P, dt, P.Fbar, &G.prof, aside ? P.side : G.stream);
-    if (e == cudaSuccess && aside) {
-      e = cudaEventRecord(P.moved, P.side);
-      if (e == cudaSuccess) e = cudaStreamWaitEvent(G.stream, P.moved, 0);
-    }
+    e = join(launch_step(P, dt, P.Fbar, &G.prof, aside ? P.side : G.stream));
     if (e != cudaSuccess) return cuda_err(e, "ibfsa_fsi_step plate");
     G.t = G.t + dt;
   }
