@@ -28,7 +28,12 @@
  *    host memory should be pinned for asynchronous copies.
  *  - Streams: every launch and copy goes to the stream given at ibfsa_create_grid (a
  *    cudaStream_t passed as void*, NULL = legacy default stream).  Calls are asynchronous
- *    unless stated; only calls returning values to the host synchronise that stream.
+ *    unless stated; only calls returning values to the host synchronise that stream.  One
+ *    exception: ibfsa_fsi_step runs the plate's step beside the fluid's last stage, on a stream
+ *    that the plate creates with the priority of the given one.  Events fork it from the given
+ *    stream and join it to it before the call returns, also with an error, so the given stream
+ *    alone orders and captures the call.  Beside a stream of a green context, and while kernel
+ *    timing is on (ibfsa_profile_enable), that step too stays on the given stream.
  *  - Layouts: state arrays are structure-of-arrays [nv][nz][ny][nx], x fastest, FP64, with
  *    nv = dim + 2 and nz = 1 in 2D.  Marker and probe arrays are [dim][n] (coordinates of point
  *    k at k, n + k, 2n + k).
@@ -310,7 +315,8 @@ int ibfsa_mlp_sample(ibfsa_grid *g, int n_max, unsigned long long seed, int atte
  * with its slope along [cos(theta0 + a), sin(theta0 + a)], a = (alpha_m/2) sin(2 pi f t + phi)
  * (Eq. 17); the slope's length stays free.  Layouts: e, v [4 (n_el + 1)] node-major; marker
  * arrays [2][n_markers].  Memory: one caller-owned workspace of ibfsa_plate_workspace_bytes(),
- * 256-byte aligned; the library allocates nothing.  Work goes to the stream given at creation;
+ * 256-byte aligned; the library allocates nothing.  Work goes to the stream given at creation
+ * (ibfsa_fsi_step: see Streams above);
  * Newton failures (iteration limit, zero or non-finite pivot, non-finite increment) set
  * IBFSA_STATUS_NOCONV, read with ibfsa_plate_get_status. */
 enum { IBFSA_PLATE_FREE = 0, IBFSA_PLATE_CLAMPED = 1 };

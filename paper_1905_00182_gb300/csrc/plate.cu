@@ -27,6 +27,7 @@
 //   implicit midpoint step: M (v_{n+1} - v_n) = dt [Q_f - Q_int(e_n + d/2)], d = e_{n+1} - e_n,
 //   Newton on d with Jacobian M + dt^2/4 dQ_int/de (both scaled by dt/2);
 //   clamp: node 0 position prescribed, slope = sigma t(t) with sigma free.
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdio.h>
@@ -688,7 +689,7 @@ struct Plate {
   int threads;
   size_t smem;
   // the structure step of a coupled step runs here, beside the fluid's last stage: it needs that
-  // stage's marker forces (forces) and is waited for before the next step (moved)
+  // stage's marker forces (forces) and is waited for before the next step (moved); NULL: in line
   cudaStream_t side = nullptr;
   cudaEvent_t forces = nullptr, moved = nullptr;
 };
@@ -757,6 +758,30 @@ static int cuda_err(cudaError_t e, const char *where) {
   char msg[256];
   snprintf(msg, sizeof(msg), "%s: %s", where, cudaGetErrorString(e));
   return api_fail(IBFSA_ERR_CUDA, msg);
+}
+
+// Whether the stream belongs to a green context, a part of the chip that the caller set aside for it
+static bool in_green_context(cudaStream_t st) {
+  typedef CUresult (*Fn)(CUstream, CUgreenCtx *);
+  void *f = nullptr;
+  cudaDriverEntryPointQueryResult q;
+  if (cudaGetDriverEntryPointByVersion("cuStreamGetGreenCtx", &f, 12040, cudaEnableDefault, &q) !=
+          cudaSuccess || q != cudaDriverEntryPointSuccess)
+    return false;
+  CUgreenCtx ctx = nullptr;
+  return reinterpret_cast<Fn>(f)(st, &ctx) == CUDA_SUCCESS && ctx;
+}
+
+// The side stream takes after the given one: its priority, and its part of the chip, which is the
+// whole one for a stream that the runtime creates: beside a stream of a green context there is none.
+static cudaError_t create_side(Plate &P) {
+  if (in_green_context(P.stream)) return cudaSuccess;
+  int priority = 0;
+  cudaError_t e = cudaStreamGetPriority(P.stream, &priority);
+  if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&P.side, cudaStreamNonBlocking, priority);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&P.forces, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&P.moved, cudaEventDisableTiming);
+  return e;
 }
 
 static void release(Plate &P) {
@@ -858,11 +883,7 @@ int ibfsa_plate_create(const ibfsa_plate_desc *desc, void *d_workspace, size_t w
   P.smem = plate::smem_doubles(desc->n_el) * sizeof(double);
   cudaError_t e = cudaFuncSetAttribute(plate::k_step, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)P.smem);
-  int least = 0, greatest = 0;  // the one-block step must not queue behind the fluid's blocks
-  if (e == cudaSuccess) e = cudaDeviceGetStreamPriorityRange(&least, &greatest);
-  if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&P.side, cudaStreamNonBlocking, greatest);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&P.forces, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&P.moved, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = create_side(P);
   if (e == cudaSuccess) e = cudaMemsetAsync(P.status, 0, 2 * sizeof(int), P.stream);
   if (e == cudaSuccess) {
     int n = (desc->n_markers > desc->n_el + 1 ? desc->n_markers : desc->n_el + 1);
@@ -996,9 +1017,10 @@ int ibfsa_fsi_step(ibfsa_grid *g, ibfsa_plate *p, double dt, int nsteps) {
   // before its convective passes: it runs beside them, on the plate's own stream (forked from and
   // joined to the grid's by events, so a capture of the grid's stream takes it along).  Its one
   // block of dependent FP64 work is then hidden: 383 x 257 in FP64, 24 elements: four steps
-  // 2.47 -> 2.06 ms; 4096 x 2048 in FP32, 40 elements: two steps 3.97 -> 3.71 ms.  With kernel
-  // timing on, everything stays on the grid's stream.
-  const bool aside = !G.prof.on;
+  // 2.47 -> 2.06 ms; 4096 x 2048 in FP32, 40 elements: two steps 3.97 -> 3.71 ms (on a stream of
+  // the greatest priority the calls of now, 1.87 and 2.84 ms, take 0.6 and 0.2 % less).  In line
+  // with kernel timing on, and where there is no side stream.
+  const bool aside = P.side && !G.prof.on;
   bool forked = false;  // work on the side stream that the grid's does not wait for yet
   // Has the grid's stream wait for the side stream; before every return, as the caller orders what
   // comes next (and ends a capture) by the grid's stream alone.  Returns the first error.

@@ -2,8 +2,10 @@
 // synchronisation, and fails the call that the caller names.  Linked with plate.cu's object file and a
 // stand-in for the stages of the grid, it shows on the CPU what ibfsa_fsi_step does with its streams.
 //
-//   fsi_streams FAIL STEPS
+//   fsi_streams FAIL STEPS PRIORITY GREEN
 //     FAIL: number of the logged call of ibfsa_fsi_step that fails (from 0; -1: none)
+//     PRIORITY: of the caller's stream; GREEN: 1 if it belongs to a green context
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdio.h>
 #include <stdlib.h>
@@ -13,7 +15,8 @@
 #include "ibfsa_internal.h"
 
 namespace {
-int g_fail = -1, g_calls = 0;
+int g_fail = -1, g_calls = 0, g_priority = 0;
+bool g_green = false;
 bool g_log = false;
 cudaError_t g_error = cudaSuccess;
 dim3 g_grid, g_block;
@@ -92,6 +95,20 @@ cudaError_t cudaStreamCreateWithPriority(cudaStream_t *s, unsigned, int priority
   printf("stream %s %d\n", name(*s).c_str(), priority);
   return cudaSuccess;
 }
+cudaError_t cudaStreamGetPriority(cudaStream_t, int *priority) {
+  *priority = g_priority;
+  return cudaSuccess;
+}
+static CUresult green_context(CUstream, CUgreenCtx *ctx) {
+  *ctx = g_green ? (CUgreenCtx)handle() : nullptr;
+  return CUDA_SUCCESS;
+}
+cudaError_t cudaGetDriverEntryPointByVersion(const char *symbol, void **f, unsigned, unsigned long long,
+                                             cudaDriverEntryPointQueryResult *r) {
+  *f = std::string(symbol) == "cuStreamGetGreenCtx" ? (void *)green_context : nullptr;
+  *r = *f ? cudaDriverEntryPointSuccess : cudaDriverEntryPointSymbolNotFound;
+  return cudaSuccess;
+}
 cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned) {
   *e = (cudaEvent_t)handle();
@@ -138,6 +155,8 @@ int main(int, char **argv) {
   if (ibfsa_plate_workspace_bytes(&d, &bytes)) return 2;
   void *ws = aligned_alloc(256, (bytes + 255) / 256 * 256);  // never read
   ibfsa_plate *p = nullptr;
+  g_priority = atoi(argv[3]);
+  g_green = atoi(argv[4]) != 0;
   if (ibfsa_plate_create(&d, ws, bytes, MAIN, &p)) return 3;
   ibfsa_grid *g = new ibfsa_grid();
   g->g.p.dim = g->g.d.dim = 2;

@@ -2,7 +2,9 @@
 CUDA runtime that only logs (fake_cudart.cpp).  Work on another stream than the caller's has to wait for
 what it reads, and the caller's stream has to wait for it: before the next step, and before the call
 returns, whatever call fails on the way (an unjoined stream leaves work that nothing orders with the
-caller's next use of the memory, and ends a capture in an error).
+caller's next use of the memory, and ends a capture in an error).  The other stream has the priority of the
+caller's, and where that belongs to a green context, whose part of the chip a stream of the runtime does
+not keep to, everything stays on the caller's.
 """
 import os
 import subprocess
@@ -29,12 +31,13 @@ def program(tmp_path_factory):
     return out
 
 
-def _run(program, fail=-1, steps=2):
-    r = subprocess.run([program, str(fail), str(steps)], capture_output=True, text=True)
+def _run(program, fail=-1, steps=2, priority=0, green=0):
+    r = subprocess.run([program, str(fail), str(steps), str(priority), str(green)], capture_output=True, text=True)
     assert r.returncode == 0, r.stderr
     lines = [x.split() for x in r.stdout.splitlines()]
     assert lines[-1][0] == "returned"
-    return [x for x in lines if x[0] != "stream"][:-1], int(lines[-1][1])
+    created = [int(x[2]) for x in lines if x[0] == "stream"]  # priorities
+    return [x for x in lines if x[0] != "stream"][:-1], int(lines[-1][1]), created
 
 
 def _reaches(log, i, stream):
@@ -58,7 +61,7 @@ def _reaches(log, i, stream):
 
 
 def test_order_of_a_coupled_step(program):
-    log, rc = _run(program)
+    log, rc, _ = _run(program)
     assert rc == 0
     work = [k for k, x in enumerate(log) if x[0] == "launch"]
     per = len(work) // 2
@@ -84,9 +87,21 @@ def test_order_of_a_coupled_step(program):
 def test_every_failure_leaves_the_streams_joined(program):
     n = len(_run(program)[0])
     for fail in range(n):
-        log, rc = _run(program, fail)
+        log, rc, _ = _run(program, fail)
         assert rc < 0
         assert sum(x[-1] == "FAILED" for x in log) == 1
         for k, x in enumerate(log):
             if x[0] == "launch" and x[-1] != "FAILED" and x[1] != "main":
                 assert _reaches(log, k, "main") is not None, (fail, k, log)
+
+
+@pytest.mark.parametrize("priority", [0, -2, -5])
+def test_side_stream_has_the_priority_given(program, priority):
+    _, rc, created = _run(program, priority=priority)
+    assert rc == 0 and created == [priority]
+
+
+def test_in_line_in_a_green_context(program):
+    log, rc, created = _run(program, green=1)
+    assert rc == 0 and created == []
+    assert len(log) == 16 and all(x[:2] == ["launch", "main"] for x in log)
