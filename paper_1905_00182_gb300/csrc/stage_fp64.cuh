@@ -452,7 +452,9 @@ __global__ void __launch_bounds__(THREADS) k_pad(Plan p, const double *__restric
     // FP32 lies within 2e-6 of the block's FP32 maximum (their relative errors, and that of
     // the threshold, stay below 3e-7, so the cell of the exact maximum is among them); the
     // other cells give 0 -- the same FP64 maxima for a fraction of the square roots.  A value
-    // beyond FP32's range gives NaN there, and its cell takes the FP64 speed.
+    // beyond FP32's range gives NaN there, and its cell takes the FP64 speed.  Sound speeds below
+    // 1.1e-19 give 0, less than 1.1e-7 of maxima of 1e-12 and more; in a block of smaller speeds
+    // every cell takes the FP64 speed.
     __shared__ float red32[3][THREADS / 32];
     const float c32 = have ? sqrtf(low_precision(c2)) : 0.f;
     float ua32[3];
@@ -470,8 +472,10 @@ __global__ void __launch_bounds__(THREADS) k_pad(Plan p, const double *__restric
       for (int w = 0; w < THREADS / 32; w++) m32[a] = fmaxf(m32[a], red32[a][w]);
     bool near = false;
 #pragma unroll
-    for (int a = 0; a < DIM; a++)
-      near |= have && !(ua32[a] + c32 < m32[a] * (1.f - 2e-6f));  // NaN counts as near
+    for (int a = 0; a < DIM; a++) {
+      const float far = m32[a] < 1e-12f ? 0.f : m32[a] * (1.f - 2e-6f);
+      near |= have && !(ua32[a] + c32 < far);  // NaN counts as near
+    }
     if (near) {
       const double c = sqrt(c2);
 #pragma unroll
