@@ -25,6 +25,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#include "fp_bits.cuh"
 #include "ibfsa_internal.h"
 #include "launch.cuh"
 #include "marker.cuh"
@@ -1438,37 +1439,6 @@ __device__ __forceinline__ float pressure_source32(const Plan &p, int dim, int i
     r2 += dx * dx;
   }
   return expf(-(float)(p.src_b * 0.693147180559945309417) * r2) * (float)p.src_scale;
-}
-
-// (double)x and (float)x (to nearest, ties to even) by integer operations and, for subnormal x, one
-// FP32 product: a conversion instruction issues at the FP64 rate, 1.8 lanes per clock and SM, so the
-// two conversions and two additions per component of the FP64 update made the last stage FP64-bound.
-// Subnormal values are common (products of small perturbations), so no case is left to the
-// instruction: it would be issued for the whole warp.
-__device__ __forceinline__ double widen(float x) {
-  const bool sub = (__float_as_uint(x) << 1) < (1u << 24);
-  const unsigned b = __float_as_uint(sub ? x * 16777216.f : x), m = b << 1;
-  const unsigned bias = sub ? 896u - 24u : m >= (255u << 24) ? 2u * 896u : 896u;
-  const unsigned hi = m ? (m >> 4) + (bias << 20) : 0u;
-  return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(b << 29));
-}
-
-__device__ __forceinline__ float narrow(double x) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const unsigned m = hi & 0x7fffffffu, e = m >> 20;
-  // the result's bits before rounding and what follows them; a carry runs into the exponent
-  unsigned f = __funnelshift_l(lo, m - (896u << 20), 3), rest = lo << 3;
-  if (e < 897u) {  // subnormal or zero
-    const unsigned full = 0x800000u | (f & 0x7fffffu), shift = 897u - e;
-    const bool some = shift <= 24u;
-    f = some ? full >> shift : 0u;
-    rest = some ? full << (32u - shift) | (rest != 0u) : 0u;
-  } else if (e > 1150u) {  // too large, infinite or not a number
-    f = m > 0x7ff00000u || (m == 0x7ff00000u && lo) ? 0x7fffffffu : 0x7f800000u;
-    rest = 0u;
-  }
-  const unsigned up = rest > 0x80000000u || (rest == 0x80000000u && (f & 1u));
-  return __uint_as_float((f + up) | (hi & 0x80000000u));
 }
 
 // The end of a stage at one cell: sponge and pressure source on the right-hand side Lc of cell

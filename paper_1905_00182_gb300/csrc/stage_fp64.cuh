@@ -15,6 +15,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#include "fp_bits.cuh"
 #include "ibfsa_internal.h"
 #include "launch.cuh"
 #include "marker.cuh"
@@ -198,18 +199,6 @@ __device__ __forceinline__ double teno5(const Plan &p, double a, double b, doubl
   const Cands k = candidates(a, b, c, d, e);
   const double *w = p.teno_w[teno_keep(k)];
   return w[0] * k.q0 + w[1] * k.q1 + w[2] * k.q2;
-}
-
-// An FP64 value as FP32 by integer operations, truncated: a conversion instruction issues at the
-// FP64 rate (1.8 per clock and SM), these at the integer rate.  Magnitudes below FP32's normal
-// range give 0, above it (and non-finite values) NaN.
-__device__ __forceinline__ float low_precision(double x) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const unsigned e = hi & 0x7ff00000u;
-  unsigned r = ((__funnelshift_l(lo, hi, 3) & 0x7fffffffu) ^ 0x40000000u) | (hi & 0x80000000u);
-  r = e < 0x38100000u ? 0u : r;
-  r = e >= 0x47f00000u ? 0x7fffffffu : r;
-  return __uint_as_float(r);
 }
 
 // TENO5 keeps every stencil when tau5 <= 4 (min beta + eps) -- each gamma_k lies in [1, 5^6], so
