@@ -116,8 +116,6 @@ void plan_geometry(const ibfsa_grid_desc &d, Plan &p) {
   p.sponge_sigma = d.sponge_sigma;
   p.alpha_pen = d.alpha_pen;
   p.beta_pen = d.beta_pen;
-  p.hprod = 1.0;
-  for (int a = 0; a < d.dim; a++) p.hprod *= p.h[a];
   // TENO5 weights of the kept stencils: d_k delta_k / sum_j d_j delta_j, d = (0.1, 0.6, 0.3)
   const double dlin[3] = {0.1, 0.6, 0.3};
   for (int m = 0; m < 8; m++) {
@@ -172,7 +170,9 @@ Layout layout_for(const ibfsa_grid_desc &d) {
   L.L = take(el * p.nv * (size_t)p.N);
   L.Qp = take(el * p.nv * (size_t)p.NP);
   L.Wp = take(el * (p.dim + 1) * (size_t)p.NP);
-  L.V = d.Re > 0.0 ? take(el * p.dim * (p.dim + 1) * (size_t)p.NB) : take(0);
+  // the FP32 form keeps its viscous fluxes on chip
+  L.V = d.Re > 0.0 && d.precision == IBFSA_FP64 ? take(el * p.dim * (p.dim + 1) * (size_t)p.NB)
+                                                : take(0);
   L.f = (d.strict_fp && d.max_markers > 0) ? take(sizeof(double) * p.dim * (size_t)p.N) : take(0);
   L.X = take(sizeof(double) * p.dim * M);
   L.U = take(sizeof(double) * p.dim * M);
@@ -309,7 +309,6 @@ int ibfsa_create_grid(const ibfsa_grid_desc *desc, void *d_workspace, size_t wor
   G.p.V = (double *)(w + L.V);
   G.p.Qp32 = (float *)(w + L.Qp);
   G.p.Wp32 = (float *)(w + L.Wp);
-  G.p.V32 = (float *)(w + L.V);
   G.p.L32 = (float *)(w + L.L);
   G.p.f = (double *)(w + L.f);
   G.X = (double *)(w + L.X);

@@ -35,7 +35,6 @@ struct Plan {
   // src_scale exp(-src_b ln2 |x - src_xc|^2), src_scale = amp cos(omega t_stage) / (gamma - 1)
   int src_on;
   double src_b, src_xc[3], src_scale;
-  double hprod;        // product of h over active directions
   // non-uniform mesh (Sec. 2): per direction, node coordinates x_i, the metric dx/dxi, 1/(dx/dxi)
   // and 1/(12 dx/dxi) at the nodes i = -NG .. n+NG-1 (stored at i + NG), FP64, and the two
   // reciprocals in FP32.  NULL: the direction is uniform with spacing h (the formulas then use
@@ -53,13 +52,13 @@ struct Plan {
   double *Qp;          // padded conservative state [nv][NP]
   double *Wp;          // padded primitives [u, v, (w), p] -> [dim+1][NP]
   double *L;           // right-hand side accumulator [nv][N]
-  double *V;           // viscous fluxes on the box [-2, n+2): [dim][dim+1][NB]
+  double *V;           // FP64 viscous fluxes on the box [-2, n+2): [dim][dim+1][NB]
   int B[3];            // box extents (n + 4 per active direction)
   long long NB;
   double *f;           // strict mode: spread force [dim][N]
   // FP32 perturbation form: the same buffers viewed as float (q - q_inf, primitive
-  // perturbations [u', v', w', p'], viscous fluxes, right-hand side)
-  float *Qp32, *Wp32, *V32, *L32;
+  // perturbations [u', v', w', p'], right-hand side; it keeps its viscous fluxes on chip)
+  float *Qp32, *Wp32, *L32;
   // the FP32 form carries the stage values of a step as FP32 increments over the FP64 state:
   // qn32 = (float)(Qn - q_inf), d1 = Q1 - Qn, d2 = Q2 - Qn
   float *qn32, *d1, *d2;
@@ -159,7 +158,7 @@ struct StageArgs {
   int stage;
   double src_scale;   // amp cos(omega t_stage) / (gamma - 1) of the pressure source (0: none)
   Prof *prof;
-  cudaEvent_t forces;  // recorded once the marker forces of the stage are known (NULL: not)
+  cudaEvent_t forces;  // 2D: recorded once the marker forces of the stage are known (NULL: not)
 };
 cudaError_t strict_stage(const Plan &p, const StageArgs &s, cudaStream_t st);
 cudaError_t fast_stage(const Plan &p, const StageArgs &s, cudaStream_t st);

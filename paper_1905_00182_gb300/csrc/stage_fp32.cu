@@ -86,22 +86,11 @@ __device__ __forceinline__ long long int_index(const Plan &p, int i, int j, int 
   return ((long long)k * p.n[1] + j) * (long long)p.n[0] + i;
 }
 
-// Peskin's four-point kernel, Eq. 11 (FP64: the IB and the probes stay in double precision)
-__device__ __forceinline__ double peskin(double r) {
-  double a = fabs(r);
-  if (a < 1.0) return (3.0 - 2.0 * a + sqrt(1.0 + 4.0 * a - 4.0 * a * a)) * 0.125;
-  if (a < 2.0) return (5.0 - 2.0 * a - sqrt(-7.0 + 12.0 * a - 4.0 * a * a)) * 0.125;
-  return 0.0;
-}
-
-// four-point supports of point k of X [dim][stride] (Eq. 10-11); *hprod (may be NULL): the
-// product of the local spacings
+// four-point supports of point k of X [dim][stride] (Eq. 10-11; FP64, as the IB and the probes)
 template <int DIM>
 __device__ __forceinline__ bool point_support(const Plan &p, const double *X, int stride, int k,
-                                              int j0[3], double w[3][4],
-                                              double *hprod = nullptr) {
+                                              int j0[3], double w[3][4]) {
   bool ok = true;
-  double hp = 1.0;
 #pragma unroll
   for (int a = 0; a < 3; a++) {
     if (a < DIM) {
@@ -111,18 +100,15 @@ __device__ __forceinline__ bool point_support(const Plan &p, const double *X, in
       } else {
         s = (X[a * stride + k] - p.lo[a]) * p.inv_h[a] - 0.5;
         j0[a] = (int)floor(s) - 1;
-        hl = p.h[a];
       }
-      hp *= hl;
 #pragma unroll
-      for (int r = 0; r < 4; r++) w[a][r] = peskin(s - (double)(j0[a] + r));
+      for (int r = 0; r < 4; r++) w[a][r] = marker::peskin4(s - (double)(j0[a] + r));
       if (j0[a] < 0 || j0[a] + 3 > p.n[a] - 1) ok = false;
     } else {
       j0[a] = 0;
       w[a][0] = 1.0; w[a][1] = 0.0; w[a][2] = 0.0; w[a][3] = 0.0;
     }
   }
-  if (hprod) *hprod = hp;
   return ok;
 }
 
@@ -2091,12 +2077,16 @@ cudaError_t run_stage(const Plan &p, const StageArgs &s, cudaStream_t st) {
     return cudaGetLastError();
   };
   // interpolation and spreading in one launch after the convective term, unless someone waits for
-  // the forces
+  // the forces (the coupled step, which is 2D)
   using Interp = std::integral_constant<int, marker::INTERP>;
   using Spread = std::integral_constant<int, marker::SPREAD>;
   using Both = std::integral_constant<int, marker::BOTH>;
-  if (s.forces && (e = markers(Interp(), K_INTERP)) != cudaSuccess) return e;
-  if (s.forces && (e = cudaEventRecord(s.forces, st)) != cudaSuccess) return e;
+  if constexpr (DIM == 2) {
+    if (s.forces && (e = markers(Interp(), K_INTERP)) != cudaSuccess) return e;
+    if (s.forces && (e = cudaEventRecord(s.forces, st)) != cudaSuccess) return e;
+  } else if (s.forces) {
+    return cudaErrorNotSupported;
+  }
   prof_begin(pr, st);
   e = launch_conv<DIM, 0, SCHEME>(p, 1, st);
   prof_end(pr, K_CONV_X, st);
@@ -2117,7 +2107,8 @@ cudaError_t run_stage(const Plan &p, const StageArgs &s, cudaStream_t st) {
     prof_end(pr, K_CONV_X, st);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  e = s.forces ? markers(Spread(), K_SPREAD) : markers(Both(), K_SPREAD);
+  if constexpr (DIM == 2) e = s.forces ? markers(Spread(), K_SPREAD) : markers(Both(), K_SPREAD);
+  else e = markers(Both(), K_SPREAD);
   if (e != cudaSuccess) return e;
   int mode = !advance ? 0 : (s.stage < 2 ? 1 : 2);
   Plan q = p;

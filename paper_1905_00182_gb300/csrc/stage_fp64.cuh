@@ -99,20 +99,12 @@ __device__ __forceinline__ double load_alpha(const Plan &p, int a) {
   return __longlong_as_double((long long)p.alpha_bits[a]);
 }
 
-// Peskin's four-point kernel, Eq. 11
-__device__ __forceinline__ double peskin(double r) {
-  double a = fabs(r);
-  if (a < 1.0) return (3.0 - 2.0 * a + sqrt(1.0 + 4.0 * a - 4.0 * a * a)) / 8.0;
-  if (a < 2.0) return (5.0 - 2.0 * a - sqrt(-7.0 + 12.0 * a - 4.0 * a * a)) / 8.0;
-  return 0.0;
-}
-
 // first of the four support nodes of position x along direction a, and their weights
 __device__ __forceinline__ int support(const Plan &p, int a, double x, double w[4]) {
   double s = divide(x - p.lo[a], p.h[a], p.inv_h[a]) - 0.5;
   int j0 = (int)floor(s) - 1;
 #pragma unroll
-  for (int r = 0; r < 4; r++) w[r] = peskin(s - (double)(j0 + r));
+  for (int r = 0; r < 4; r++) w[r] = marker::peskin4(s - (double)(j0 + r));
   return j0;
 }
 
@@ -1141,14 +1133,11 @@ __global__ void __launch_bounds__(THREADS) k_visc_div(Plan p) {
 // ------------------------------------------------------------------------------------------
 // immersed boundary (Eq. 7-9)
 // ------------------------------------------------------------------------------------------
-// the four-point supports of point k of X [dim][nm] in every direction (Eq. 10-11); *hprod
-// (may be NULL) receives the product of the local spacings, h^d of the delta at the point
+// the four-point supports of point k of X [dim][nm] in every direction (Eq. 10-11)
 template <int DIM>
 __device__ __forceinline__ bool marker_support(const Plan &p, const double *X, int nm, int k,
-                                               int j0[3], double w[3][4],
-                                               double *hprod = nullptr) {
+                                               int j0[3], double w[3][4]) {
   bool ok = true;
-  double hp = 1.0;
 #pragma unroll
   for (int a = 0; a < 3; a++) {
     if (a < DIM) {
@@ -1156,11 +1145,9 @@ __device__ __forceinline__ bool marker_support(const Plan &p, const double *X, i
         double s, hl;
         j0[a] = mesh::support_stretched(p, a, X[a * nm + k], &s, &hl);
 #pragma unroll
-        for (int r = 0; r < 4; r++) w[a][r] = peskin(s - (double)(j0[a] + r));
-        hp *= hl;
+        for (int r = 0; r < 4; r++) w[a][r] = marker::peskin4(s - (double)(j0[a] + r));
       } else {
         j0[a] = support(p, a, X[a * nm + k], w[a]);
-        hp *= p.h[a];
       }
       if (j0[a] < 0 || j0[a] + 3 > p.n[a] - 1) ok = false;
     } else {
@@ -1168,7 +1155,6 @@ __device__ __forceinline__ bool marker_support(const Plan &p, const double *X, i
       w[a][0] = 1.0; w[a][1] = 0.0; w[a][2] = 0.0; w[a][3] = 0.0;
     }
   }
-  if (hprod) *hprod = hp;
   return ok;
 }
 
@@ -1199,7 +1185,7 @@ __device__ __forceinline__ void strict_supports(const Plan &p, int k0,
         sx = divide(x - p.lo[a], p.h[a], p.inv_h[a]) - 0.5;
         j = (int)floor(sx) - 1;
       }
-      sw[m][a][q] = peskin(sx - (double)(j + q));
+      sw[m][a][q] = marker::peskin4(sx - (double)(j + q));
       if (q == 0) {
         sj[m][a] = j;
         shl[m][a] = hl;
@@ -1656,7 +1642,7 @@ cudaError_t run_stage(const Plan &p, const StageArgs &s, cudaStream_t st) {
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   int advance = s.stage >= 0;
   // Markers.  Strict: interpolation now, spreading after the viscous term.  Fast: both in one launch
-  // after the convective term, unless someone waits for the forces.
+  // after the convective term, unless someone waits for the forces (the coupled step, which is 2D).
   using Interp = std::integral_constant<int, marker::INTERP>;
   using Spread = std::integral_constant<int, marker::SPREAD>;
   using Both = std::integral_constant<int, marker::BOTH>;
@@ -1678,8 +1664,11 @@ cudaError_t run_stage(const Plan &p, const StageArgs &s, cudaStream_t st) {
     prof_end(pr, part() == marker::INTERP ? K_INTERP : K_SPREAD, st);
     return es != cudaSuccess ? es : cudaGetLastError();
   };
-  if ((STRICT || s.forces) && (e = markers(Interp())) != cudaSuccess) return e;
-  if (s.forces && (e = cudaEventRecord(s.forces, st)) != cudaSuccess) return e;
+  if (DIM > 2 && s.forces) return cudaErrorNotSupported;
+  if constexpr (STRICT || DIM == 2) {
+    if ((STRICT || s.forces) && (e = markers(Interp())) != cudaSuccess) return e;
+    if (s.forces && (e = cudaEventRecord(s.forces, st)) != cudaSuccess) return e;
+  }
   prof_begin(pr, st);
   e = launch_conv<DIM, 0, SCHEME>(p, 1, st);
   prof_end(pr, K_CONV_X, st);
@@ -1703,7 +1692,8 @@ cudaError_t run_stage(const Plan &p, const StageArgs &s, cudaStream_t st) {
   // strict: the viscous divergence into L, then the spreading; fast: the spreading, then the
   // divergence as part of finish
   if constexpr (!STRICT) {
-    e = s.forces ? markers(Spread()) : markers(Both());
+    if constexpr (DIM == 2) e = s.forces ? markers(Spread()) : markers(Both());
+    else e = markers(Both());
     if (e != cudaSuccess) return e;
   }
   const bool viscous = p.Re > 0.0;
