@@ -1392,8 +1392,9 @@ __global__ void __launch_bounds__(128) k_markers(Plan p, const double *__restric
                                                  double Bc, double dt, int advance) {
   begin_kernel();
   constexpr int C = marker::Support<DIM, G>::C;
-  const int r = threadIdx.x % G, km = (int)((blockIdx.x * blockDim.x + threadIdx.x) / G);
-  const int k = min(km, p.nm - 1), M = p.max_markers;
+  const int r = threadIdx.x % G, M = p.max_markers;
+  const unsigned km = blockIdx.x * (blockDim.x / G) + threadIdx.x / G, nm = (unsigned)p.nm;
+  const int k = (int)min(km, nm - 1);
   const auto t = marker::support<DIM, G>(p, p.X, M, k, r);
   const long long s = pad_index(p, t.c0[0], t.c0[1], t.c0[2]);
   double F[DIM];
@@ -1410,7 +1411,7 @@ __global__ void __launch_bounds__(128) k_markers(Plan p, const double *__restric
 #pragma unroll
     for (int a = 0; a < DIM; a++) acc[a] = marker::group_sum<G>(acc[a] * t.wr);
     double mine = 0.0;
-    if (km < p.nm) {
+    if (km < nm) {
       if (t.ok) mine = marker::force<DIM>(p, k, r, acc, xis, xin, xio, A, Bc, dt, advance);
       else marker::off_grid<DIM>(p, k, r, xin, xio, advance);
     }
@@ -1418,7 +1419,7 @@ __global__ void __launch_bounds__(128) k_markers(Plan p, const double *__restric
     for (int a = 0; a < DIM; a++) F[a] = __shfl_sync(0xffffffffu, mine, a, G);
   }
   if constexpr (!(PART & marker::SPREAD)) return;
-  if (km >= p.nm || !t.ok) return;
+  if (km >= nm || !t.ok) return;
   const long long o = int_index(p, t.c0[0], t.c0[1], t.c0[2]);
   const double sc = t.wr * (p.dS[k] * t.ihp);
   double f[DIM];
