@@ -757,8 +757,10 @@ __global__ void __launch_bounds__(THREADS) k_conv_char(Plan p, int first) {
 }
 
 
-// Component-wise: a tile is 32 lines (y for A = 0, consecutive x otherwise) by up to 8 K faces of
-// one component; a warp takes the 32 lines of K consecutive faces.  The kernel is bound by the
+// Component-wise: a tile is 32 lines by up to 8 K faces of one component; a warp takes the 32 lines of
+// K consecutive faces.  The lines are consecutive in x (A > 0) or the rows of a plane (A = 0).  With JOIN
+// they are segments of rows, numbered through y, z and then the segments, so that lanes are idle in the
+// last tile only (100000 x 4: 4 lanes of 32 without); a line's place is then looked up, ~2 us a pass.  The kernel is bound by the
 // FP64 pipe (1.7 lanes per clock and SM, so a warp instruction costs its SM quarter ~75 cycles):
 // what counts is FP64 operations, and that every SM quarter has several warps to issue them from.
 // Hence K faces per thread, whose differences are shared (faces_of_line), a block per component
@@ -779,7 +781,7 @@ struct LineTile {
   static constexpr size_t BYTES = sizeof(double) * (2 * LEN * R + (FACES + 1) * R);
 };
 
-template <int DIM, int A, int SCHEME, int K>
+template <int DIM, int A, int SCHEME, int K, bool JOIN>
 __global__ void __launch_bounds__(THREADS, 3) k_conv(Plan p, int first, int nseg) {
   begin_kernel();
   constexpr int NV = DIM + 2;
@@ -794,25 +796,44 @@ __global__ void __launch_bounds__(THREADS, 3) k_conv(Plan p, int first, int nseg
   double *sh = sfm + T::LEN * T::R;   // face fluxes
   const double alpha = load_alpha(p, A);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  constexpr int LN = A == 0 ? 1 : 0;  // direction of the tile's lines
-
   const int c = blockIdx.x % NV;                    // component
   const int segl = (p.n[A] + nseg - 1) / nseg;
-  const int seg0 = (blockIdx.x / NV % nseg) * segl;  // first cell along A
-  const int line0 = blockIdx.x / (NV * nseg) * T::R;
-  const int other = blockIdx.y;
-  const int ncell = min(segl, p.n[A] - seg0);
-  if (ncell <= 0) return;
-  const int nface = ncell + 1, nst = ncell + 6, nrow = min(T::R, p.n[LN] - line0);
-  int I[3] = {0, 0, 0};
-  I[A] = seg0;
-  I[LN] = line0;
-  if (DIM > 2) I[3 - A - LN] = other;
+  // first cell along A, cells of the tile (JOIN: of its longest line) and its lines; offsets of its
+  // first staged and its first own cell
+  int seg0 = 0, ncell = segl, nrow, pad0 = 0, int0 = 0;
+  // JOIN: the same of every line
+  __shared__ int line_seg0[JOIN ? T::R : 1], line_ncell[JOIN ? T::R : 1];
+  __shared__ int line_pad0[JOIN ? T::R : 1], line_int0[JOIN ? T::R : 1];
+  constexpr int LN = A == 0 ? 1 : 0;  // direction of the tile's lines
   const long long stp[3] = {1, p.P[0], (long long)p.P[0] * p.P[1]};
   const long long sti[3] = {1, p.n[0], (long long)p.n[0] * p.n[1]};
-  const double *Qb = p.Qp + pad_index(p, I[0], I[1], I[2]) - 3 * stp[A];
-  const double *Wb = p.Wp + pad_index(p, I[0], I[1], I[2]) - 3 * stp[A];
-  double *Lb = p.L + int_index(p, I[0], I[1], I[2]);
+  if constexpr (JOIN) {
+    static_assert(A == 0, "rows along x");
+    const unsigned rows = (unsigned)(p.n[1] * p.n[2]), first_line = blockIdx.x / NV * T::R;
+    nrow = (int)min((unsigned)T::R, rows * nseg - first_line);
+    if (warp == 0) {
+      const unsigned line = first_line + min(lane, nrow - 1), seg = line / rows, row = line - seg * rows;
+      const int z = (int)(row / p.n[1]), y = (int)row - z * p.n[1], x = (int)seg * segl;
+      line_seg0[lane] = x;
+      line_ncell[lane] = min(segl, p.n[0] - x);  // 0 or less: an empty last segment
+      line_pad0[lane] = (int)(pad_index(p, x, y, z) - 3);
+      line_int0[lane] = (int)int_index(p, x, y, z);
+    }
+    __syncthreads();
+  } else {
+    seg0 = (blockIdx.x / NV % nseg) * segl;
+    const int line0 = blockIdx.x / (NV * nseg) * T::R;
+    ncell = min(segl, p.n[A] - seg0);
+    if (ncell <= 0) return;
+    nrow = min(T::R, p.n[LN] - line0);
+    int I[3] = {0, 0, 0};
+    I[A] = seg0;
+    I[LN] = line0;
+    if (DIM > 2) I[3 - A - LN] = blockIdx.y;
+    pad0 = (int)(pad_index(p, I[0], I[1], I[2]) - 3 * stp[A]);
+    int0 = (int)int_index(p, I[0], I[1], I[2]);
+  }
+  const int nface = ncell + 1, nst = ncell + 6;
 
   // the slots a warp's last faces read beyond the staged cells hold zeros
   for (int l = nst - 1 + warp; l < T::LEN; l += THREADS / 32) {
@@ -826,13 +847,14 @@ __global__ void __launch_bounds__(THREADS, 3) k_conv(Plan p, int first, int nseg
     const int e = threadIdx.x + i * THREADS;
     const int l = A == 0 ? e % nst : e / T::R, row = A == 0 ? e / nst : e % T::R;
     if (l >= nst || row >= nrow) continue;
-    const int go = (int)(row * stp[LN] + l * stp[A]);
-    const double q = Qb[c * p.NP + go];
+    if (JOIN && l >= line_ncell[row] + 6) continue;
+    const int go = JOIN ? line_pad0[row] + l : pad0 + (int)(row * stp[LN] + l * stp[A]);
+    const double q = p.Qp[c * p.NP + go];
     double F;
     if (c == 0) {
-      F = Qb[(1 + A) * p.NP + go];
+      F = p.Qp[(1 + A) * p.NP + go];
     } else {
-      const double ua = Wb[A * p.NP + go], pr = Wb[DIM * p.NP + go];
+      const double ua = p.Wp[A * p.NP + go], pr = p.Wp[DIM * p.NP + go];
       if (c == NV - 1) {
         F = (q + pr) * ua;
       } else {
@@ -850,7 +872,7 @@ __global__ void __launch_bounds__(THREADS, 3) k_conv(Plan p, int first, int nseg
   // 2. faces m+1/2, m = seg0 - 1 + fi: f+ of staged cells fi .. fi+4, f- of fi+1 .. fi+5
   const int fi0 = warp * K;  // this warp's first face
   if (fi0 < nface) {
-    const int at = min(lane, nrow - 1) * T::SR + fi0 * T::SL;
+    const int line = min(lane, nrow - 1), at = line * T::SR + fi0 * T::SL;
     double f[K + 4], h[K], g[K];
 #pragma unroll
     for (int j = 0; j < K + 4; j++) f[j] = sfp[at + j * T::SL];
@@ -859,7 +881,9 @@ __global__ void __launch_bounds__(THREADS, 3) k_conv(Plan p, int first, int nseg
     for (int j = 0; j < K + 4; j++) f[j] = sfm[at + j * T::SL];
     fail |= faces_of_line<SCHEME, true, K>(p, f, g) << K;
     if constexpr (SCHEME == IBFSA_TENO5) {
-      const unsigned some = (1u << min(K, nface - fi0)) - 1;  // slots that hold a face
+      // slots that hold a face
+      const int faces = (JOIN ? line_ncell[line] + 1 : nface) - fi0;
+      const unsigned some = (1u << max(0, min(K, faces))) - 1;
       fail &= some | some << K;
       // full TENO5 where the sufficient test failed: each lane walks its own failed stencils
       // (re-read from shared memory), one copy of the code
@@ -888,13 +912,14 @@ __global__ void __launch_bounds__(THREADS, 3) k_conv(Plan p, int first, int nseg
   for (int i = 0; i < (A == 0 ? T::R / NW : (T::FACES + NW - 1) / NW); i++) {
     const int row = A == 0 ? warp + i * NW : lane, l = A == 0 ? lane : warp + i * NW;
     if (l >= ncell || row >= nrow) continue;
+    if (JOIN && l >= line_ncell[row]) continue;
     const double *hh = sh + row * T::HR + l * T::HL;
     const double dh = hh[T::HL] - hh[0];
-    const int ia = seg0 + l;
+    const int ia = (JOIN ? line_seg0[row] : seg0) + l;
     constexpr double half = FOLD ? 0.5 : 1.0;
     const bool str = p.mm[A] != nullptr;
     const double inv = half * (str ? p.minv[A][ia + NG] : p.inv_h[A]);
-    double *Lc = Lb + c * p.N + row * sti[LN] + l * sti[A];
+    double *Lc = p.L + c * p.N + (JOIN ? line_int0[row] + l : int0 + row * sti[LN] + l * sti[A]);
     const double prev = first ? 0.0 : *Lc;
     if (char_cell(p, A, ia)) *Lc = prev;
     else if (STRICT) *Lc = prev - divide(dh, str ? p.mm[A][ia + NG] : p.h[A], inv);
@@ -1587,47 +1612,68 @@ cudaError_t launch_conv_char(const Plan &p, int first, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-// Faces per thread of k_conv: the K whose tiles (rowtiles: lines / 32 x components) give the
-// smallest (tiles of the busiest SM) x (FP64 operations of a tile), the tiles of a line being as
-// equal as they can be.  A face costs ~2 (4 + (K + 3)/K) + 1 operations, a staged cell ~3.
-// Measured, TENO5: 256^3, a y pass 3.47 / 3.82 / 4.91 ms with K = 4 / 2 / 1; WENO5-JS at 256^2,
-// where 31-cell tiles give 1.9 blocks per SM, 70 / 73 / 80 us; TENO5 at 383 x 257, x pass 59 / 50
-// / 54 us.
-inline int conv_faces(long long rowtiles, int n, int *nseg) {
-  int best = 4;
+// The tiles of a pass of k_conv.  Faces per thread: the K whose tiles give the smallest (tiles of the
+// busiest SM) x (FP64 operations of a tile), the tiles of a line being as equal as they can be.  A
+// face costs ~2 (4 + (K + 3)/K) + 1 operations, a staged cell ~3.  Measured, TENO5: 256^3, a y pass
+// 3.47 / 3.82 / 4.91 ms with K = 4 / 2 / 1; WENO5-JS at 256^2, where 31-cell tiles give 1.9 blocks
+// per SM, 70 / 73 / 80 us; TENO5 at 383 x 257, x pass 59 / 50 / 54 us.
+// Joined rows along x where that saves an eighth of more than two tiles per SM, the whole step
+// without / with: WENO5-JS, 100000 x 4 7.59 / 2.67 ms, strict 19.7 / 6.46, 300 x 33 x 33 3.74 / 3.07,
+// strict 9.59 / 7.78; one tile per SM or less, 16 x 16 96 / 104 us, 65 x 65 108 / 111.
+struct ConvTiles {
+  int K, nseg;
+  bool join;
+  long long tiles;  // of one component
+};
+
+template <int DIM, int A>
+inline ConvTiles conv_tiles(const Plan &p) {
+  const int n = p.n[A];
+  ConvTiles best{};
   double cost = -1.0;
   for (int K = 4; K >= 1; K /= 2) {
     const int most = 8 * K - 1, ns = (n + most - 1) / most, seg = (n + ns - 1) / ns;
+    const long long across = A == 0 ? (long long)((p.n[1] + 31) / 32) * p.n[2]
+                                    : (long long)((p.n[0] + 31) / 32) * p.n[A == 1 ? 2 : 1];
+    const long long joined = ((long long)p.n[1] * p.n[2] * ns + 31) / 32;
+    const bool join = A == 0 && (DIM + 2) * across * ns > 2 * 152 && 8 * joined <= 7 * across * ns;
+    const long long tiles = join ? joined : across * ns;
     const double tile = (seg + 1) * (9.0 + 2.0 * (K + 3) / K) + 3.0 * (seg + 6) + 2.0 * seg;
-    const double c = (double)((rowtiles * ns + 151) / 152) * tile;
+    const double c = (double)(((DIM + 2) * tiles + 151) / 152) * tile;
     if (cost < 0.0 || c < cost) {
       cost = c;
-      best = K;
-      *nseg = ns;
+      best = {K, ns, join, tiles};
     }
   }
   return best;
 }
 
-template <int DIM, int A, int SCHEME, int K>
-cudaError_t launch_conv_k(const Plan &p, int first, int nseg, long long tiles, cudaStream_t st) {
+template <int DIM, int A, int SCHEME, int K, bool JOIN>
+cudaError_t launch_conv_k(const Plan &p, int first, const ConvTiles &t, cudaStream_t st) {
   constexpr size_t smem = LineTile<A, K>::BYTES;
-  static_assert(smem <= 48 * 1024, "within the default dynamic shared memory");
+  static_assert(smem <= 47 * 1024, "with the lines' places within the default shared memory");
   static_assert(LineTile<A, K>::FACES <= 32, "the update walks a line of cells with one warp");
-  dim3 grid((unsigned)((DIM + 2) * tiles * nseg), A == 2 ? p.n[1] : p.n[2]);
-  launch(k_conv<DIM, A, SCHEME, K>, grid, THREADS, smem, st, p, first, nseg);
+  const int planes = JOIN ? 1 : p.n[A == 2 ? 1 : 2];
+  dim3 grid((unsigned)((DIM + 2) * (t.tiles / planes)), planes);
+  launch(k_conv<DIM, A, SCHEME, K, JOIN>, grid, THREADS, smem, st, p, first, t.nseg);
   return cudaGetLastError();
+}
+
+template <int DIM, int A, int SCHEME, int K>
+cudaError_t launch_conv_k(const Plan &p, int first, const ConvTiles &t, cudaStream_t st) {
+  if constexpr (A == 0)
+    if (t.join) return launch_conv_k<DIM, A, SCHEME, K, true>(p, first, t, st);
+  return launch_conv_k<DIM, A, SCHEME, K, false>(p, first, t, st);
 }
 
 template <int DIM, int A, int SCHEME>
 cudaError_t launch_conv(const Plan &p, int first, cudaStream_t st) {
   if (p.charwise) return launch_conv_char<DIM, A, SCHEME>(p, first, st);
-  const long long tiles = (p.n[A == 0 ? 1 : 0] + 31) / 32;
-  int nseg = 1;
-  switch (conv_faces((DIM + 2) * tiles * (A == 2 ? p.n[1] : p.n[2]), p.n[A], &nseg)) {
-    case 4: return launch_conv_k<DIM, A, SCHEME, 4>(p, first, nseg, tiles, st);
-    case 2: return launch_conv_k<DIM, A, SCHEME, 2>(p, first, nseg, tiles, st);
-    default: return launch_conv_k<DIM, A, SCHEME, 1>(p, first, nseg, tiles, st);
+  const ConvTiles t = conv_tiles<DIM, A>(p);
+  switch (t.K) {
+    case 4: return launch_conv_k<DIM, A, SCHEME, 4>(p, first, t, st);
+    case 2: return launch_conv_k<DIM, A, SCHEME, 2>(p, first, t, st);
+    default: return launch_conv_k<DIM, A, SCHEME, 1>(p, first, t, st);
   }
 }
 
