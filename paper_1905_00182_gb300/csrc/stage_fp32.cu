@@ -102,7 +102,7 @@ __device__ __forceinline__ bool point_support(const Plan &p, const double *X, in
         j0[a] = (int)floor(s) - 1;
       }
 #pragma unroll
-      for (int r = 0; r < 4; r++) w[a][r] = marker::peskin4(s - (double)(j0[a] + r));
+      for (int r = 0; r < 4; r++) w[a][r] = marker::peskin(s - (double)(j0[a] + r));
       if (j0[a] < 0 || j0[a] + 3 > p.n[a] - 1) ok = false;
     } else {
       j0[a] = 0;

@@ -104,7 +104,7 @@ __device__ __forceinline__ int support(const Plan &p, int a, double x, double w[
   double s = divide(x - p.lo[a], p.h[a], p.inv_h[a]) - 0.5;
   int j0 = (int)floor(s) - 1;
 #pragma unroll
-  for (int r = 0; r < 4; r++) w[r] = marker::peskin4(s - (double)(j0 + r));
+  for (int r = 0; r < 4; r++) w[r] = marker::peskin(s - (double)(j0 + r));
   return j0;
 }
 
@@ -1173,7 +1173,7 @@ __device__ __forceinline__ bool marker_support(const Plan &p, const double *X, i
         double s, hl;
         j0[a] = mesh::support_stretched(p, a, X[a * nm + k], &s, &hl);
 #pragma unroll
-        for (int r = 0; r < 4; r++) w[a][r] = marker::peskin4(s - (double)(j0[a] + r));
+        for (int r = 0; r < 4; r++) w[a][r] = marker::peskin(s - (double)(j0[a] + r));
       } else {
         j0[a] = support(p, a, X[a * nm + k], w[a]);
       }
@@ -1213,7 +1213,7 @@ __device__ __forceinline__ void strict_supports(const Plan &p, int k0,
         sx = divide(x - p.lo[a], p.h[a], p.inv_h[a]) - 0.5;
         j = (int)floor(sx) - 1;
       }
-      sw[m][a][q] = marker::peskin4(sx - (double)(j + q));
+      sw[m][a][q] = marker::peskin(sx - (double)(j + q));
       if (q == 0) {
         sj[m][a] = j;
         shl[m][a] = hl;
