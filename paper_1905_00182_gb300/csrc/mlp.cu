@@ -174,7 +174,7 @@ __global__ void __launch_bounds__(32 * TRAIN_WARPS, TRAIN_BLOCKS)
             float *__restrict__ loss) {
   __shared__ __align__(16) unsigned char img[STAGED_BYTES];
   __shared__ __align__(16) unsigned char tiles_of[TRAIN_WARPS][TILE_BYTES];
-  stage_image(img, gimg);
+  stage_image<true>(img, gimg);
   __syncthreads();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
   // this warp's share: units 16 (w/2).. x inputs 16 (w%2).. of dW3 and dW2; half w%2 of dW1
@@ -355,7 +355,7 @@ __global__ void __launch_bounds__(256) k_eval(const unsigned char *__restrict__ 
                                               float *__restrict__ omega, float inv_n,
                                               float *__restrict__ loss) {
   __shared__ __align__(16) unsigned char img[STAGED_BYTES];
-  stage_image(img, gimg);
+  stage_image<false>(img, gimg);
   __syncthreads();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
   const int warps = blockDim.x >> 5;

@@ -37,12 +37,12 @@ constexpr int PACKED_BYTES = 11264;
 constexpr int LD8 = 8, LD32 = 40;
 constexpr int S_W1 = 0;                  // [32][8]
 constexpr int S_W4T = 512;               // [32][8]
-constexpr int S_W2 = 1024;               // [32][40]
+constexpr int S_W2 = 1024;               // [32][40], and on in the image's order
 constexpr int S_W3 = S_W2 + 2560;        // [32][40]
-constexpr int S_W2T = S_W3 + 2560;       // [32][40]
+constexpr int S_W4 = S_W3 + 2560;        // [8][40]
+constexpr int S_W2T = S_W4 + 640;        // [32][40]
 constexpr int S_W3T = S_W2T + 2560;      // [32][40]
-constexpr int S_W4 = S_W3T + 2560;       // [8][40]
-constexpr int S_B1 = S_W4 + 640;         // [32] f32
+constexpr int S_B1 = S_W3T + 2560;       // [32] f32, and on as in the image
 constexpr int S_B2 = S_B1 + 128;
 constexpr int S_B3 = S_B2 + 128;
 constexpr int S_B4 = S_B3 + 128;         // [8] f32
@@ -96,31 +96,20 @@ __device__ __forceinline__ float ldb(const unsigned char *img, int off, int i) {
   return reinterpret_cast<const float *>(img + off)[i];
 }
 
-// the image's shared copy; a barrier has to follow
+// the image's shared copy, with BACK the transposed matrices too; a barrier has to follow
+template <bool BACK>
 __device__ __forceinline__ void stage_image(unsigned char *img,
                                             const unsigned char *__restrict__ gimg) {
-  constexpr int CHUNKS = PACKED_BYTES / 16;
-  for (int i = threadIdx.x; i < CHUNKS; i += blockDim.x) {
-    const int b = 16 * i;
-    int to;
-    if (b < OFF_W2) {
-      if (i & 1) continue;
-      to = S_W1 + b / 2;
-    } else if (b < OFF_W2T) {  // W2, W3, W4: rows of 64 bytes
-      const int r = (b - OFF_W2) / 64;
-      to = (r < 32 ? S_W2 + 80 * r : r < 64 ? S_W3 + 80 * (r - 32) : S_W4 + 80 * (r - 64)) + b % 64;
-    } else if (b < OFF_W4T) {  // W2T, W3T
-      const int r = (b - OFF_W2T) / 64;
-      to = S_W2T + 80 * r + (b - OFF_W2T) % 64;
-    } else if (b < OFF_B1) {
-      if (i & 1) continue;
-      to = S_W4T + (b - OFF_W4T) / 2;
-    } else {
-      if (b >= OFF_B4 + 32) continue;
-      to = S_B1 + (b - OFF_B1);
-    }
-    *reinterpret_cast<uint4 *>(img + to) = reinterpret_cast<const uint4 *>(gimg)[i];
-  }
+  auto chunk = [&](int to, int from) {
+    *reinterpret_cast<uint4 *>(img + to) = *reinterpret_cast<const uint4 *>(gimg + from);
+  };
+  constexpr int ROWS = BACK ? 136 : 72;  // of 64 bytes: W2, W3, W4 (, W2T, W3T)
+  for (int i = threadIdx.x; i < 4 * ROWS; i += blockDim.x)
+    chunk(S_W2 + 80 * (i >> 2) + 16 * (i & 3), OFF_W2 + 16 * i);
+  if (threadIdx.x < 32) chunk(S_W1 + 16 * threadIdx.x, OFF_W1 + 32 * threadIdx.x);
+  else if (threadIdx.x < 58) chunk(S_B1 + 16 * (threadIdx.x - 32), OFF_B1 + 16 * (threadIdx.x - 32));
+  else if (BACK && threadIdx.x >= 64 && threadIdx.x < 96)
+    chunk(S_W4T + 16 * (threadIdx.x - 64), OFF_W4T + 32 * (threadIdx.x - 64));
 }
 
 // 16x32 hidden layer: acc[j][.] (n-tile j = units 8j..8j+7) = bias + A(16 x K) W^T
