@@ -249,20 +249,34 @@ def measured_peaks():
         return {"hbm_gbs": HBM_FALLBACK_GBS}, "fallback"
 
 
+# the sources that the stage's kernels of a form are compiled from
+STAGE_SOURCES = {
+    "fp32": ("stage_fp32.cu", "fp_bits.cuh", "ibfsa_internal.h", "launch.cuh", "marker.cuh",
+             "mesh.cuh", "mlp_tile.cuh", "tma.cuh"),
+    "fp64": ("stage_fp64.cuh", "stage_fp64_fast.cu", "fp_bits.cuh", "ibfsa_internal.h",
+             "launch.cuh", "marker.cuh", "mesh.cuh"),
+}
+
+
+def source_sha(precision):
+    h = hashlib.sha256()
+    for name in STAGE_SOURCES[precision]:
+        with open(os.path.join(ROOT, "paper_1905_00182_gb300", "csrc", name), "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:16]
+
+
 def ncu_traffic(kernel_class, precision):
     """DRAM bytes per launch from the committed ncu summary, if it was taken on the current
-    kernel source (else None)."""
+    kernel sources (else None)."""
     path = os.path.join(ROOT, "profiles", "traffic.json")
     try:
         with open(path) as f:
             rec = json.load(f)
     except (OSError, ValueError):
         return None
-    name = "stage_fp32.cu" if precision == "fp32" else "stage_fp64.cuh"
-    src = os.path.join(ROOT, "paper_1905_00182_gb300", "csrc", name)
-    sha = hashlib.sha256(open(src, "rb").read()).hexdigest()[:16]
     ent = rec.get(f"{precision}:{kernel_class}")
-    if not ent or ent.get("source_sha") != sha:
+    if not ent or ent.get("source_sha") != source_sha(precision):
         return None
     return ent.get("bytes_per_launch_full")
 
