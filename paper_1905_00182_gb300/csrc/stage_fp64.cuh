@@ -803,7 +803,8 @@ __global__ void __launch_bounds__(THREADS, 3) k_conv(Plan p, int first, int nseg
   const int segl = (p.n[A] + nseg - 1) / nseg;
   // first cell along A, cells of the tile (JOIN: of its longest line) and its lines; offsets of its
   // first staged and its first own cell
-  int seg0 = 0, ncell = segl, nrow, pad0 = 0, int0 = 0;
+  int seg0 = 0, ncell = segl, nrow;
+  long long pad0 = 0, int0 = 0;
   // JOIN: the same of every line
   __shared__ int line_seg0[JOIN ? T::R : 1], line_ncell[JOIN ? T::R : 1];
   __shared__ int line_pad0[JOIN ? T::R : 1], line_int0[JOIN ? T::R : 1];
@@ -833,9 +834,11 @@ __global__ void __launch_bounds__(THREADS, 3) k_conv(Plan p, int first, int nseg
     I[A] = seg0;
     I[LN] = line0;
     if (DIM > 2) I[3 - A - LN] = blockIdx.y;
-    pad0 = (int)(pad_index(p, I[0], I[1], I[2]) - 3 * stp[A]);
-    int0 = (int)int_index(p, I[0], I[1], I[2]);
+    pad0 = pad_index(p, I[0], I[1], I[2]) - 3 * stp[A];
+    int0 = int_index(p, I[0], I[1], I[2]);
   }
+  const double *Qb = p.Qp + pad0, *Wb = p.Wp + pad0;
+  double *Lb = p.L + int0;
   const int nface = ncell + 1, nst = ncell + 6;
 
   // the slots a warp's last faces read beyond the staged cells hold zeros
@@ -851,13 +854,13 @@ __global__ void __launch_bounds__(THREADS, 3) k_conv(Plan p, int first, int nseg
     const int l = A == 0 ? e % nst : e / T::R, row = A == 0 ? e / nst : e % T::R;
     if (l >= nst || row >= nrow) continue;
     if (JOIN && l >= line_ncell[row] + 6) continue;
-    const int go = JOIN ? line_pad0[row] + l : pad0 + (int)(row * stp[LN] + l * stp[A]);
-    const double q = p.Qp[c * p.NP + go];
+    const int go = JOIN ? line_pad0[row] + l : (int)(row * stp[LN] + l * stp[A]);
+    const double q = Qb[c * p.NP + go];
     double F;
     if (c == 0) {
-      F = p.Qp[(1 + A) * p.NP + go];
+      F = Qb[(1 + A) * p.NP + go];
     } else {
-      const double ua = p.Wp[A * p.NP + go], pr = p.Wp[DIM * p.NP + go];
+      const double ua = Wb[A * p.NP + go], pr = Wb[DIM * p.NP + go];
       if (c == NV - 1) {
         F = (q + pr) * ua;
       } else {
@@ -922,7 +925,7 @@ __global__ void __launch_bounds__(THREADS, 3) k_conv(Plan p, int first, int nseg
     constexpr double half = FOLD ? 0.5 : 1.0;
     const bool str = p.mm[A] != nullptr;
     const double inv = half * (str ? p.minv[A][ia + NG] : p.inv_h[A]);
-    double *Lc = p.L + c * p.N + (JOIN ? line_int0[row] + l : int0 + row * sti[LN] + l * sti[A]);
+    double *Lc = Lb + c * p.N + (JOIN ? line_int0[row] + l : row * sti[LN] + l * sti[A]);
     const double prev = first ? 0.0 : *Lc;
     if (char_cell(p, A, ia)) *Lc = prev;
     else if (STRICT) *Lc = prev - divide(dh, str ? p.mm[A][ia + NG] : p.h[A], inv);
