@@ -95,7 +95,7 @@ typedef struct {
   int scheme;              /* IBFSA_WENO5JS | IBFSA_TENO5 | IBFSA_MLP_TENO5 */
   int precision;           /* IBFSA_FP64 | IBFSA_FP32_PERTURB */
   int strict_fp;           /* 1: every FP64 operation rounded separately (no fused
-                              multiply-add), divisions kept as divisions, spreading summed
+                              multiply-add), quotients rounded as divisions, spreading summed
                               cell by cell in marker order -- the result is reproducible bit
                               for bit by a sequential FP64 evaluation of the same formulas in
                               the same order.  0: fused multiply-add and reciprocals allowed,

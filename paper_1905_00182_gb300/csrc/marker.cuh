@@ -2,17 +2,16 @@
 // lanes, for the immersed-boundary kernels whose sums need no fixed order (FP32 form, fast FP64).
 //
 // A group of 16 lanes owns one marker, lane r in 3D the row of four support cells along x at (y, z)
-// offsets (r & 3, r >> 2), in 2D the cell (r & 3, r >> 2); many 2D markers take 4 lanes each, lane
-// r the row at y offset r.  What bounds these kernels is the FP64 pipe (1.7 lanes per clock and
+// offsets (r & 3, r >> 2), in 2D the cell (r & 3, r >> 2); many 2D markers take 4 lanes each, lane r
+// the row at y offset r.  What bounds these kernels is the FP64 pipe (1.7 lanes per clock and
 // SM): a warp instruction costs ~75 cycles whatever its active lanes, so the 4 DIM kernel weights
 // are evaluated one per lane and exchanged, each row is summed by its lane, and only the rows' sums
 // are reduced by shuffles.  Few lanes per marker are fewer instructions in all, many a shorter chain:
 // 16 lanes in 2D while every quarter of an SM gets at most two warps.
-// Before, with one thread per marker for the interpolation (a chain of 64 divisions in 3D) and the
-// weights of a marker evaluated by each of its 64 threads for the FP64 spreading (event times,
-// ~4 us of them the launch): FP32 form, 20000 markers in 3D: interpolation 108 -> 70 us, spreading
-// 88 -> 62 us; 1500 markers: 70 -> 14 and 12 -> 13 us; FP64, 5000 markers: 43 -> 18 and 169 ->
-// 22 us; 2D, 1024 markers (FP32): 26 -> 13 and 10 -> 12 us.
+// Interpolation and spreading together (event times, ~4 us a launch), against one thread per marker
+// for the interpolation (a chain of 64 divisions in 3D) and, in FP64, the weights of a marker
+// evaluated by each of its 64 threads for the spreading: FP32 form, 20000 markers in 3D 196 -> 98 us,
+// 1500 82 -> 18; FP64, 5000 in 3D 212 -> 28; 2D, 1024 (FP32) 36 -> 12.
 #pragma once
 
 #include "ibfsa_internal.h"
@@ -170,10 +169,11 @@ enum Part { INTERP = 1, SPREAD = 2, BOTH = 3 };
 // calls f(G) with the lanes per marker for nm markers, an integral_constant
 template <int DIM, typename F>
 inline void with_group(int nm, F f) {
-  if (DIM > 2 || nm <= 2 * 4 * 152 * 2)
-    f(std::integral_constant<int, 16>());
-  else
-    f(std::integral_constant<int, (DIM > 2 ? 16 : 4)>());
+  if constexpr (DIM == 2) {
+    // with 16 lanes (two markers a warp) more than two warps for each quarter of an SM
+    if (nm > 2 * 4 * 152 * 2) return f(std::integral_constant<int, 4>());
+  }
+  f(std::integral_constant<int, 16>());
 }
 
 }  // namespace marker

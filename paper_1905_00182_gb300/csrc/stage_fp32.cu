@@ -216,18 +216,19 @@ __device__ __forceinline__ float2 f2(float v) { return make_float2(v, v); }
 // of the faces after staged cells i+2, i+3: the .x lanes are the f+ stencils upwind to downwind,
 // the .y lanes the f- stencils downwind to upwind, so one load per k fetches both sides.  First
 // differences, second differences and their squares are taken once for both faces (each face by
-// itself: 26 packed operations, the pair: 41; the passes are bound by instruction issue).  At 512^3
-// with TENO5 x 2.27 -> 1.97 ms, y and z 2.36 -> 2.22 ms; WENO5-JS at 2048^2, before one side and
-// component at a time without packing, x 95 -> 67 us, y 101 -> 70 us.  With the f- stencil reversed, the packed indicator
-// of z0 z1 z2 is (beta_0+, beta_2-) and that of z2 z3 z4 is (beta_2+, beta_0-) (the squares are
-// symmetric under the reversal), so tau5 and the all-kept test are those of each side; the
-// linear combination takes per-lane coefficient pairs.
+// itself: 26 packed operations, the pair: 41; the passes are bound by instruction issue).  Pairs for
+// single faces: TENO5 at 512^3 x 2.27 -> 1.97 ms, y and z 2.36 -> 2.22 ms (1.78, 1.99 and 2.02 since
+// k_conv32_x and the exchange of k_conv32_tma); WENO5-JS at 2048^2, single faces not packed, x 95 ->
+// 67 us, y 101 -> 70 us (65 and 63 since).  With the f- stencil reversed, the packed indicator of
+// z0 z1 z2 is (beta_0+, beta_2-) and that of z2 z3 z4 is (beta_2+, beta_0-) (the squares are
+// symmetric under the reversal), so tau5 and the all-kept test are those of each side; the linear
+// combination takes per-lane coefficient pairs.
 //
 // TENO5: the all-kept test is scale-invariant, so the indicators are taken times 4, (13/3) t^2 +
-// u^2, of twice the split flux (STAGE_SCALE), with the floor 16e-30.  The linear (all-kept) result is computed without branches; only
-// when some lane of the warp has a side that cuts a stencil does the whole warp enter the full
-// TENO5 (a uniform branch, no divergence to reconverge): every lane of the warp must call it, and
-// v0, v1 say which of its faces exist.
+// u^2, of twice the split flux (STAGE_SCALE), with the floor 16e-30.  The linear (all-kept) result
+// is computed without branches; only when some lane of the warp has a side that cuts a stencil does
+// the whole warp enter the full TENO5 (a uniform branch, no divergence to reconverge): every lane of
+// the warp must call it, and v0, v1 say which of its faces exist.
 // WENO5-JS: weights d_k / (eps + beta_k)^2 over their common denominator, the reconstruction as
 // the middle value plus a weighted mean of the candidates' differences from it.
 template <int SCHEME, int K>
@@ -261,8 +262,10 @@ __device__ __forceinline__ void faces_pz(const Plan &tw, const float2 (&z)[K + 4
       lin = __ffma2_rn(make_float2(-3.f / 60.f, 2.f / 60.f), z[j + 4], lin);
       h[j] = lin.x + lin.y;
       if (__any_sync(0xffffffffu, (j ? v1 : v0) && !(kx && ky))) {
-        const float hx = kx ? lin.x : teno5<4>(tw, z[j].x, z[j + 1].x, z[j + 2].x, z[j + 3].x, z[j + 4].x);
-        const float hy = ky ? lin.y : teno5<4>(tw, z[j + 4].y, z[j + 3].y, z[j + 2].y, z[j + 1].y, z[j].y);
+        const float hx = kx ? lin.x : teno5<4>(tw, z[j].x, z[j + 1].x, z[j + 2].x, z[j + 3].x,
+                                               z[j + 4].x);
+        const float hy = ky ? lin.y : teno5<4>(tw, z[j + 4].y, z[j + 3].y, z[j + 2].y, z[j + 1].y,
+                                               z[j].y);
         h[j] = hx + hy;
       }
     } else {
@@ -277,8 +280,8 @@ __device__ __forceinline__ void faces_pz(const Plan &tw, const float2 (&z)[K + 4
       const float2 n2 = __ffma2_rn(make_float2(12.f / 60.f, -5.f / 60.f), d[j + 2],
                                    __fmul2_rn(make_float2(-3.f / 60.f, 2.f / 60.f), d[j + 3]));
       const float2 num = __ffma2_rn(p2, n2, __ffma2_rn(p1, n1, __fmul2_rn(p0, n0)));
-      const float2 den = __ffma2_rn(make_float2(0.3f, 0.1f), p2,
-                                    __ffma2_rn(f2(0.6f), p1, __fmul2_rn(make_float2(0.1f, 0.3f), p0)));
+      const float2 d01 = __ffma2_rn(f2(0.6f), p1, __fmul2_rn(make_float2(0.1f, 0.3f), p0));
+      const float2 den = __ffma2_rn(make_float2(0.3f, 0.1f), p2, d01);
       h[j] = (z[j + 2].x + __fdividef(num.x, den.x)) + (z[j + 2].y + __fdividef(num.y, den.y));
     }
   }
@@ -640,9 +643,13 @@ __device__ __forceinline__ void roe_eigen32(const Free &fs, const float wl[DIM +
 // network tiles.  The characteristic-wise option: four blocks for y and z, three for x (85
 // registers; four there spill and are 6 % slower); with one (138 registers, and each stencil
 // loaded and projected with the eigenvectors' zeros, field by field) a pass over 160 x 144 x 150
-// took 432 / 559 / 543 us, now 226 / 211 / 203 us.  The x pass gives each warp one row of the tile.
+// took 432 / 559 / 543 us, now 213 / 191 / 181 us.  The x pass gives each warp one row of the tile.
+constexpr int conv32_blocks(int a, int scheme, bool chr) {
+  return scheme == IBFSA_MLP_TENO5 ? 4 : chr ? (a == 0 ? 3 : 4) : 6;
+}
+
 template <int DIM, int A, int SCHEME, bool CHAR = false>
-__global__ void __launch_bounds__(THREADS, SCHEME == IBFSA_MLP_TENO5 ? 4 : (CHAR ? (A == 0 ? 3 : 4) : 6))
+__global__ void __launch_bounds__(THREADS, conv32_blocks(A, SCHEME, CHAR))
     k_conv32(Plan p, int first) {
   begin_kernel();
   constexpr int NV = DIM + 2;
@@ -744,8 +751,8 @@ __global__ void __launch_bounds__(THREADS, SCHEME == IBFSA_MLP_TENO5 ? 4 : (CHAR
   // the thread's face slot ps (row >= nrow or fi >= nface: none).  Learned weights along x: the
   // tile's existing faces are numbered through its rows, so that a short last tile fills a few warps
   // (the network costs a warp the same for one face as for 32): at 128^3, where the third tile of a
-  // row holds 2 of its 63 cells, the pass takes 868 us
-  // (1038 with the slots numbered through all 64 places of a row).
+  // row holds 2 of its 63 cells, the pass takes 870 us (1038 with the slots numbered through all 64
+  // places of a row).
   const unsigned face_magic = 65536u / nface + 1;  // e / nface for e < 512, nface <= 64
   auto face_of = [&](int ps, int &row, int &fi) {
     const int e = threadIdx.x + ps * THREADS;
@@ -923,7 +930,8 @@ struct RowTile {
 };
 
 template <int DIM, int SCHEME, int LPR>
-__global__ void __launch_bounds__(THREADS, SCHEME == IBFSA_TENO5 ? 5 : 6) k_conv32_x(Plan p, int seg, int nseg) {
+__global__ void __launch_bounds__(THREADS, SCHEME == IBFSA_TENO5 ? 5 : 6)
+    k_conv32_x(Plan p, int seg, int nseg) {
   begin_kernel();
   constexpr int NV = DIM + 2;
   using T = RowTile<DIM, LPR>;
@@ -1003,7 +1011,8 @@ __global__ void __launch_bounds__(THREADS, SCHEME == IBFSA_TENO5 ? 5 : 6) k_conv
   if (!own || l >= ncell) return;
   const bool two = l + 1 < ncell;
   const float inv0 = char_cell(p, 0, i) ? 0.f : FLUX_SCALE<SCHEME> * mesh::inv32(p, 0, i);
-  const float inv1 = !two || char_cell(p, 0, i + 1) ? 0.f : FLUX_SCALE<SCHEME> * mesh::inv32(p, 0, i + 1);
+  const float inv1 =
+      !two || char_cell(p, 0, i + 1) ? 0.f : FLUX_SCALE<SCHEME> * mesh::inv32(p, 0, i + 1);
   float *L = p.L32 + (size_t)(row0 + row) * p.n[0] + i;
   const bool pair = two && !(p.n[0] & 1);  // 8-byte stores: rows and segments start at even cells
 #pragma unroll
@@ -1635,8 +1644,9 @@ __global__ void __launch_bounds__(THREADS, 4) k_visc_finish32(Plan p, const floa
 }
 
 // 3D viscous term + finish, marching along z.  A 32 x 8 block of threads owns 32 x 8 columns
-// and walks a z-chunk of zc planes (chosen by march_chunk): velocity perturbations of five planes (x, y halo 4) sit in a shared-
-// memory ring, refilled from registers loaded one plane ahead; at each plane c the 9 gradients
+// and walks a z-chunk of zc planes (chosen by march_chunk): velocity perturbations of five planes
+// (x, y halo 4) sit in a shared-memory ring, refilled from registers loaded one plane ahead; at each
+// plane c the 9 gradients
 // are evaluated at the block's cells and at the x/y halo points the x/y divergence needs,
 // giving F_v,x and F_v,y (shared memory, divergence taken at once) and F_v,z, whose
 // z-differences are accumulated per thread into the cells c-2 .. c+2 of its column; cell c-2
@@ -2010,21 +2020,21 @@ cudaError_t launch_conv(const Plan &p, int first, cudaStream_t st) {
     }
   }
   if constexpr (A != 0 || SCHEME == IBFSA_MLP_TENO5) {
-  constexpr size_t smem =
-      conv_smem<DIM, A>() + (SCHEME == IBFSA_MLP_TENO5 ? (size_t)mlp::PACKED_BYTES : 0);
-  e = cudaFuncSetAttribute(k_conv32<DIM, A, SCHEME>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem);
-  if (e != cudaSuccess) return e;
-  dim3 grid;
-  if (A == 0) {
-    grid = dim3((p.n[0] + T::SEG - 1) / T::SEG, (p.n[1] + T::ROWS - 1) / T::ROWS, p.n[2]);
-  } else {
-    int nseg = (p.n[A] + T::SEG - 1) / T::SEG;
-    int nx = (p.n[0] + T::ROWS - 1) / T::ROWS;
-    grid = dim3(nseg * nx, A == 1 ? p.n[2] : p.n[1]);
-  }
-  launch(k_conv32<DIM, A, SCHEME>, grid, THREADS, smem, st, p, first);
-  return cudaGetLastError();
+    constexpr size_t smem =
+        conv_smem<DIM, A>() + (SCHEME == IBFSA_MLP_TENO5 ? (size_t)mlp::PACKED_BYTES : 0);
+    e = cudaFuncSetAttribute(k_conv32<DIM, A, SCHEME>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)smem);
+    if (e != cudaSuccess) return e;
+    dim3 grid;
+    if (A == 0) {
+      grid = dim3((p.n[0] + T::SEG - 1) / T::SEG, (p.n[1] + T::ROWS - 1) / T::ROWS, p.n[2]);
+    } else {
+      int nseg = (p.n[A] + T::SEG - 1) / T::SEG;
+      int nx = (p.n[0] + T::ROWS - 1) / T::ROWS;
+      grid = dim3(nseg * nx, A == 1 ? p.n[2] : p.n[1]);
+    }
+    launch(k_conv32<DIM, A, SCHEME>, grid, THREADS, smem, st, p, first);
+    return cudaGetLastError();
   }
 }
 

@@ -1,7 +1,7 @@
 // stage_fp64.cuh -- FP64 kernels of one Runge-Kutta stage of the IB-WENO/TENO method
 // (arXiv:1905.00182, Sec. 2).  Included twice: once with IBFSA_STRICT = 1 and --fmad=false
-// (every operation rounded separately, in the order the formulas are written below, divisions
-// kept, spreading summed in marker order), once with IBFSA_STRICT = 0 (fused multiply-add,
+// (every operation rounded separately, in the order the formulas are written below, quotients
+// rounded as divisions, spreading summed in marker order), once with IBFSA_STRICT = 0 (fused multiply-add,
 // reciprocals, atomic spreading).
 //
 // Per stage:  pad (ghosts + primitives + split speeds)  ->  IB interpolation and penalty force
@@ -760,20 +760,21 @@ __global__ void __launch_bounds__(THREADS) k_conv_char(Plan p, int first) {
 }
 
 
-// Component-wise: a tile is 32 lines by up to 8 K faces of one component; a warp takes the 32 lines of
-// K consecutive faces.  The lines are consecutive in x (A > 0) or the rows of a plane (A = 0).  With JOIN
-// they are segments of rows, numbered through y, z and then the segments, so that lanes are idle in the
-// last tile only (100000 x 4: 4 lanes of 32 without); a line's place is then looked up, ~2 us a pass.  The kernel is bound by the
-// FP64 pipe (1.7 lanes per clock and SM, so a warp instruction costs its SM quarter ~75 cycles):
-// what counts is FP64 operations, and that every SM quarter has several warps to issue them from.
-// Hence K faces per thread, whose differences are shared (faces_of_line), a block per component
-// (the split fluxes of one take 27 KB; a small grid has five times the blocks), segments of equal
-// length instead of a short last one, idle lanes only in whole warps, and a K chosen by the
-// launcher (conv_faces): 4 on large grids, less where tiles of 31 cells would leave SMs idle.
+// Component-wise: a tile is 32 lines by up to 8 K faces of one component; a warp takes the 32 lines
+// of K consecutive faces.  The lines are consecutive in x (A > 0) or the rows of a plane (A = 0).
+// With JOIN they are segments of rows, numbered through y, z and then the segments, so that lanes
+// are idle in the last tile only (100000 x 4: 4 lanes of 32 work without); a line's place is then
+// looked up, ~2 us a pass.  The kernel is bound by the FP64 pipe (1.7 lanes per clock and SM, so a
+// warp instruction costs its SM quarter ~75 cycles): what counts is FP64 operations, and that every
+// SM quarter has several warps to issue them from.  Hence K faces per thread, whose differences are
+// shared (faces_of_line), a block per component (the split fluxes of one take 27 KB; a small grid has
+// five times the blocks), segments of equal length instead of a short last one, idle lanes only in
+// whole warps, and a K chosen by the launcher (conv_tiles): 4 on large grids, less where tiles of 31
+// cells would leave SMs idle.
 // Against one face per thread on tiles of 63 (x) or 15 (y, z) cells with all components staged:
-// TENO5 at 256^3 x 8.06 -> 3.53 ms, y and z 5.92 -> 3.47 ms (FP64 operations per cell of a pass,
+// TENO5 at 256^3 x 8.06 -> 3.53 ms, y and z 5.92 -> 3.48 ms (FP64 operations per cell of a pass,
 // counted by ncu at 192^3 with K = 2: 121, before ~300 in x); WENO5-JS at 256^2 x 138 -> 70 us,
-// y 92 -> 70 us; strict TENO5 at 61 x 53 x 47 x 620 -> 242 us, y and z 961 -> 220 us.
+// y 92 -> 70 us; strict TENO5 at 61 x 53 x 47 x 620 -> 225 us (joined), y and z 961 -> 212 us.
 template <int A, int K>
 struct LineTile {
   static constexpr int R = 32;                      // lines
@@ -1288,7 +1289,7 @@ __global__ void k_ib_interp(Plan p, const double *__restrict__ xis, const double
 // marker order (a ballot per 256 markers), and each cell takes those that cover it.  The table's
 // bounding box lets the blocks away from the body write their zeros at once.  One block walking
 // the markers one after the other (each waiting for the weights and the read-modify-write of its
-// cells) took 12 us per marker: 400 markers 4720 us, this 77 us.
+// cells) took 12 us per marker: 400 markers 4720 us, table and gather 74 us.
 struct SpreadTable {
   double *w;     // [12][n] weights (direction, offset)
   double *hp;    // [n] product of the local spacings
