@@ -1,8 +1,8 @@
 // stage_fp64.cuh -- FP64 kernels of one Runge-Kutta stage of the IB-WENO/TENO method
 // (arXiv:1905.00182, Sec. 2).  Included twice: once with IBFSA_STRICT = 1 and --fmad=false
 // (every operation rounded separately, in the order the formulas are written below, quotients
-// rounded as divisions, spreading summed in marker order), once with IBFSA_STRICT = 0 (fused multiply-add,
-// reciprocals, atomic spreading).
+// rounded as divisions, spreading summed in marker order), once with IBFSA_STRICT = 0 (fused
+// multiply-add, reciprocals, atomic spreading).
 //
 // Per stage:  pad (ghosts + primitives + split speeds)  ->  IB interpolation and penalty force
 //   (Eq. 7-8)  ->  convective flux differences x, y, z  ->  viscous fluxes and their divergence
@@ -602,7 +602,7 @@ __global__ void __launch_bounds__(THREADS) k_conv_char(Plan p, int first) {
   } else {
     const unsigned nseg = (p.n[A] + T::SEG - 1) / T::SEG;
     // blocks start in the order of x, y: the line tiles slowest, so that the short last ones, which
-    // take less time, come after all full ones (33^3, nine passes: 6.4 -> 5.9 ms)
+    // take less time, come after all full ones (33^3, a step: 2.13 -> 1.95 ms)
     const unsigned id = blockIdx.y * gridDim.x + blockIdx.x, rest = id / nseg;
     seg0 = (int)(id % nseg) * T::SEG;
     line0 = (int)(rest / gridDim.y) * T::ROWS;  // x of the first line
@@ -817,7 +817,8 @@ __global__ void __launch_bounds__(THREADS, 3) k_conv(Plan p, int first, int nseg
     const unsigned rows = (unsigned)(p.n[1] * p.n[2]), first_line = blockIdx.x / NV * T::R;
     nrow = (int)min((unsigned)T::R, rows * nseg - first_line);
     if (warp == 0) {
-      const unsigned line = first_line + min(lane, nrow - 1), seg = line / rows, row = line - seg * rows;
+      const unsigned line = first_line + min(lane, nrow - 1), seg = line / rows;
+      const unsigned row = line - seg * rows;
       const int z = (int)(row / p.n[1]), y = (int)row - z * p.n[1], x = (int)seg * segl;
       line_seg0[lane] = x;
       line_ncell[lane] = min(segl, p.n[0] - x);  // 0 or less: an empty last segment
@@ -1602,9 +1603,9 @@ inline unsigned blocks_for(long long n, int threads) {
 
 // One block keeps an SM's FP64 pipe busy.  With few blocks one at a time per SM is faster (more than
 // half of its shared memory asked for): the next one starts where a block ends, instead of two or
-// three that take long (TENO5's full evaluation) on one SM beside SMs that are done.  TENO5, nine
-// passes with 5 blocks per SM and fewer / with as many as fit: 33^3 5.9 / 8.9 ms, 56^3 16.2 / 17.7,
-// 64^3 23.4 / 25.1, 64 x 48 x 40 12.1 / 11.8; above, 100^3 87.8 / 85.7, 1021 x 771 23.8 / 23.1.
+// three that take long (TENO5's full evaluation) on one SM beside SMs that are done.  TENO5, a step
+// one at a time up to 5 blocks per SM / as many as fit: 33^3 1.95 / 2.96 ms, 56^3 5.4 / 5.9, 64^3
+// 7.8 / 8.4, 64 x 48 x 40 4.09 / 3.91; with more blocks 100^3 29.3 / 28.6, 1021 x 771 7.9 / 7.7.
 template <int DIM, int A, int SCHEME>
 cudaError_t launch_conv_char(const Plan &p, int first, cudaStream_t st) {
   using T = ConvTile<A>;
